@@ -89,9 +89,14 @@ typedef struct {
                              prefix scan of bit masks, re-run from each accepted
                              move that changes E_Delta (L % 4 == 0, 4 <= L <= 64;
                              other sizes fall back to MUCA_RES_GLOBAL) */
-#define MUCA_RES_BONDS 5  /* the disordered model's kernel (muca_set_bonds): one thread
-                             per walker, couplings per bond; reported by
-                             muca_get_config, not selectable in muca_options */
+#define MUCA_RES_BONDS 5  /* the disordered model (muca_set_bonds): couplings per bond;
+                             reported by muca_get_config, not selectable in
+                             muca_options */
+#define MUCA_RES_ROWS 6   /* spins in HBM/L2, one lane per site of a row (or of a
+                             segment of it), the row's decisions iterated together
+                             until they reproduce themselves (3 <= L <= 64): the
+                             choice of MUCA_RES_AUTO; reported by muca_get_config,
+                             not selectable in muca_options */
 
 /* debug_flags bits */
 #define MUCA_DEBUG_TALLY_CHECK 1 /* recompute E_J, E_Delta, M after every sweep call */

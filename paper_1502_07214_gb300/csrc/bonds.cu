@@ -14,14 +14,9 @@
 // that leave the window through zero thresholds, the histogram after every
 // sweep, the recorded series) is the clean model's.
 //
-// One thread per walker, a warp of 8 to 32 walkers (about four warps per SM);
-// the walkers of a warp read whole 32-byte sectors per packed spin word.  One
-// kernel per row length: for L % 4 == 0 a walker's row lives in registers
-// (bonds_rows: x neighbours are byte extracts, the y / z neighbour words are
-// loaded once per packed word, a site's six couplings are one load of its
-// pack), for other L every neighbour and coupling is read from global memory
-// (bonds_sites).  Each site keeps one dependent chain: its left neighbour,
-// the field, the threshold load from the table, the compare.
+// This kernel serves L = 2, whose rows are too short for the site-per-lane
+// kernel (rows.cu runs every other size, with the same table): one thread per
+// walker, every neighbour and coupling read from global memory.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -101,81 +96,6 @@ __device__ __forceinline__ void bonds_sites(const GroupDev &g, uint32_t *lat, ui
     }
 }
 
-__device__ __forceinline__ int sbyte(uint32_t w, int q) { return (int)(int8_t)(uint8_t)(w >> (8 * q)); }
-__device__ __forceinline__ int jbyte(unsigned long long w, int k)
-{
-    return (int)(int8_t)(uint8_t)(w >> (8 * k));
-}
-
-// One sweep of one walker with rows of L = 4 LW sites: the row held in
-// registers (every index a compile-time constant), the y / z neighbour words
-// of each packed word loaded once for its four sites, the six couplings of a
-// site from one load of its pack, the row stored once at its end.  Site
-// order, Philox words and thresholds are those of bonds_sites: with
-// L % 4 == 0 the block of site i = row L + 4 j + q is row LW + j and its
-// word is q.
-template <int LW>
-__device__ __forceinline__ void bonds_rows(const GroupDev &g, uint32_t *lat, uint32_t key0,
-                                           uint32_t seed, uint64_t sw, int &EJ, int &ED, int &M)
-{
-    constexpr int L = 4 * LW;
-    const int nj = 24 * g.jmax + 1, off = 12 * g.jmax;
-    const unsigned long long *__restrict__ J6 = g.J6;
-    const uint32_t *__restrict__ thrJ = g.thrJ;
-    const ptrdiff_t st = g.Wpad;
-    const uint32_t slo = (uint32_t)sw, shi = (uint32_t)(sw >> 32);
-    auto wp = [&](int row, int j) { return lat + ((ptrdiff_t)row * LW + j) * st; };
-    for (int z = 0; z < L; ++z) {
-        const int zm = z == 0 ? L - 1 : z - 1, zp = z + 1 == L ? 0 : z + 1;
-        for (int y = 0; y < L; ++y) {
-            const int ym = y == 0 ? L - 1 : y - 1, yp = y + 1 == L ? 0 : y + 1;
-            const int row = z * L + y;
-            uint32_t O[LW];
-#pragma unroll
-            for (int j = 0; j < LW; ++j) O[j] = *wp(row, j);
-            const unsigned long long *jrow = J6 + (ptrdiff_t)row * L;
-#pragma unroll
-            for (int j = 0; j < LW; ++j) {
-                // the y / z neighbour words of this word (not changed by the row)
-                const uint32_t YMj = *wp(z * L + ym, j), YPj = *wp(z * L + yp, j);
-                const uint32_t ZMj = *wp(zm * L + y, j), ZPj = *wp(zp * L + y, j);
-                const uint4 rn =
-                    philox4x32_10(make_uint4((uint32_t)(row * LW + j), slo, shi, 0u), key0, seed);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int x = 4 * j + q;
-                    constexpr int kL = L;
-                    const int xr = x + 1 == kL ? 0 : x + 1, xl = x == 0 ? kL - 1 : x - 1;
-                    const uint32_t word = q == 0 ? rn.x : q == 1 ? rn.y : q == 2 ? rn.z : rn.w;
-                    const unsigned long long jj = __ldg(jrow + x);
-                    const int h = jbyte(jj, 0) * sbyte(O[xr >> 2], xr & 3) +
-                                  jbyte(jj, 1) * sbyte(O[xl >> 2], xl & 3) +
-                                  jbyte(jj, 2) * sbyte(YPj, q) + jbyte(jj, 3) * sbyte(YMj, q) +
-                                  jbyte(jj, 4) * sbyte(ZPj, q) + jbyte(jj, 5) * sbyte(ZMj, q);
-                    const int s = sbyte(O[j], q);
-                    const int lo = (s == -1) ? 0 : -1, hi = (s == 1) ? 0 : 1;
-                    const int sp = (word >> 31) ? hi : lo;
-                    const int d = sp * sp - s * s;
-                    const int dEJ = -(sp - s) * h;
-                    const uint32_t thr =
-                        __ldg(thrJ + ((ptrdiff_t)(ED - g.e_min) * 3 + (d + 1)) * nj + dEJ + off);
-                    if ((word & 0x7FFFFFFFu) < thr) {
-                        O[j] = (O[j] & ~(0xFFu << (8 * q))) | ((uint32_t)(uint8_t)sp << (8 * q));
-                        EJ += dEJ;
-                        ED += d;
-                        M += sp - s;
-                    }
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < LW; ++j) *wp(row, j) = O[j];
-        }
-    }
-}
-
-// One kernel per row kind: LW > 0 the rows of L = 4 LW sites (bonds_rows),
-// LW = 0 any L (bonds_sites); each gets its own register allocation.
-template <int LW>
 __global__ void __launch_bounds__(32)
 sweep_bonds_kernel(const GroupDev *__restrict__ groups, const BlockDesc *__restrict__ blocks,
                    uint32_t seed, uint64_t sweep0, int n_sweeps, int64_t ts_pos, int record)
@@ -192,10 +112,7 @@ sweep_bonds_kernel(const GroupDev *__restrict__ groups, const BlockDesc *__restr
     int EJ = g.tal[w], ED = g.tal[g.Wpad + w], M = g.tal[2 * g.Wpad + w];
     for (int k = 0; k < n_sweeps; ++k) {
         const uint64_t sw = sweep0 + (uint64_t)k;
-        if constexpr (LW > 0)
-            bonds_rows<LW>(g, lat, key0, seed, sw, EJ, ED, M);
-        else
-            bonds_sites(g, lat, key0, seed, sw, EJ, ED, M);
+        bonds_sites(g, lat, key0, seed, sw, EJ, ED, M);
         hist_inc(g.hist, ED - g.e_min, amask);
         if (record) {
             int32_t *o = g.ts + (ts_pos + k) * 3 * (int64_t)g.W + w;
@@ -211,40 +128,13 @@ sweep_bonds_kernel(const GroupDev *__restrict__ groups, const BlockDesc *__restr
 
 }  // namespace
 
-cudaError_t launch_sweeps_bonds(int L, const GroupDev *groups_dev, const BlockDesc *blocks_dev,
+cudaError_t launch_sweeps_bonds(const GroupDev *groups_dev, const BlockDesc *blocks_dev,
                                 int n_blocks, uint32_t seed, uint64_t sweep0, int n_sweeps,
                                 int64_t ts_pos, bool record, cudaStream_t st)
 {
     if (n_blocks <= 0) return cudaSuccess;
-    const int rec = record ? 1 : 0;
-    switch (L % 4 == 0 ? L : 0) {
-#define MUCA_BOND_LAUNCH(LL)                                                                 \
-    case LL:                                                                                 \
-        sweep_bonds_kernel<LL / 4><<<n_blocks, 32, 0, st>>>(groups_dev, blocks_dev, seed,     \
-                                                            sweep0, n_sweeps, ts_pos, rec);  \
-        break;
-        MUCA_BOND_LAUNCH(4)
-        MUCA_BOND_LAUNCH(8)
-        MUCA_BOND_LAUNCH(12)
-        MUCA_BOND_LAUNCH(16)
-        MUCA_BOND_LAUNCH(20)
-        MUCA_BOND_LAUNCH(24)
-        MUCA_BOND_LAUNCH(28)
-        MUCA_BOND_LAUNCH(32)
-        MUCA_BOND_LAUNCH(36)
-        MUCA_BOND_LAUNCH(40)
-        MUCA_BOND_LAUNCH(44)
-        MUCA_BOND_LAUNCH(48)
-        MUCA_BOND_LAUNCH(52)
-        MUCA_BOND_LAUNCH(56)
-        MUCA_BOND_LAUNCH(60)
-        MUCA_BOND_LAUNCH(64)
-#undef MUCA_BOND_LAUNCH
-        default:
-            sweep_bonds_kernel<0><<<n_blocks, 32, 0, st>>>(groups_dev, blocks_dev, seed, sweep0,
-                                                           n_sweeps, ts_pos, rec);
-            break;
-    }
+    sweep_bonds_kernel<<<n_blocks, 32, 0, st>>>(groups_dev, blocks_dev, seed, sweep0, n_sweeps,
+                                                ts_pos, record ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -9,11 +9,11 @@ namespace muca {
 
 // Packed acceptance table of one group, as the sweep kernel reads it: one
 // allocation of table_rows(nE) rows of kRow uint32 (160 bytes):
-//   rows 0 .. kGuard-1     zero (guard)
-//   row kGuard + e         E_Delta = e_min + e, e = 0 .. nE-1, every move kind:
+//   rows 0 .. kPad+kGuard-1  zero (guard)
+//   row kPad + kGuard + e  E_Delta = e_min + e, e = 0 .. nE-1, every move kind:
 //     column 13 (d + 1) + (d == 0 ? (dE_J + 12) / 2 : dE_J + 6),
 //     d = -1: s = +-1 -> 0, d = 0: s = +-1 -> -+1, d = +1: s = 0 -> +-1
-//   last kGuard rows       zero (guard)
+//   last kGuard+kPad rows  zero (guard)
 // The d = 0 columns repeat in every row so that one index formula serves all
 // moves.  The guard rows let the kernel read the rows E_Delta +- 1 and copy
 // windows of rows without bounds checks; they are never compared against
@@ -21,20 +21,33 @@ namespace muca {
 constexpr int kRow = 40;
 constexpr int kBlk = 13;
 constexpr int kGuard = 2;
-inline size_t table_rows(int nE) { return (size_t)nE + 2 * kGuard; }
+// The site-per-lane kernel (rows.cu) reads, for decisions that it will not
+// keep, rows up to 32 below or above a walker's E_Delta: kPad further rows of
+// zeros lie before and after a table's rows (the disordered model's table,
+// which has no guard rows, included).
+constexpr int kPad = 32;
+inline size_t table_rows(int nE) { return (size_t)nE + 2 * (kGuard + kPad); }
 
 // Spin layout of a group: int8 spins packed four consecutive sites of a row
 // per 32-bit word, walker-minor: word (row, j) of walker w is at
 //   spins[(row * Lw + j) * Wpad + w],  row = y + L z,  Lw = ceil(L / 4),
 // and byte q of that word is site x = 4 j + q (bytes past x = L - 1 are 0).
-// The 32 lanes of a warp thus read 128 contiguous bytes per word.
+// The 32 lanes of a warp thus read 128 contiguous bytes per word.  Groups that
+// the site-per-lane kernel sweeps (rows.cu) keep the same words walker by
+// walker instead, word (row, j) of walker w at
+//   spins[w * L * L * rw + row * rw + j],
+// rows of rw >= Lw words (the words past Lw are 0), so that the lanes of a row
+// read consecutive bytes.  Either way word (row, j) of walker w is
+//   spins[(row * rw + j) * wstr + w * cstr].
 
 // Per-group parameters in device memory.
 struct GroupDev {
     int L, V, W, Wpad, Lw;      // linear size, sites, walkers, padded walker stride, words/row
     int e_min, nE;              // E_Delta window start and number of bins
     uint32_t walker0;           // global id of walker 0 (Philox key word 0)
-    uint32_t *spins;            // [L * L][Lw][Wpad] packed words
+    uint32_t *spins;            // packed words, strides wstr (word) and cstr (walker)
+    int64_t wstr, cstr;         // in words: (Wpad, 1), or (1, L * L * rw) walker by walker
+    int rw;                     // words per row: Lw, or more walker by walker
     int32_t *tal;               // [3][Wpad]: E_J, E_Delta, M
     unsigned long long *hist;   // [nE]
     const uint32_t *thrE;       // the row of E_Delta = e_min in the table allocation
@@ -86,8 +99,8 @@ cudaError_t prepare_global_kernel(size_t smem_bytes);
 // BlockDesc.S walker slots, a power of 2 in [4, 32]).  Two instantiations:
 // rows of up to kWsNarrowMaxL sites (wide = false) and longer rows.
 constexpr int kWsNarrowMaxL = 32;
-// kernel kinds: lanes, shared tile, split narrow, split wide, row scan,
-// disordered model
+// kernel kinds with block lists: lanes, shared tile, split narrow, split wide,
+// row scan, disordered model (L = 2)
 constexpr int kKinds = 6;
 cudaError_t launch_sweeps_ws(const GroupDev *groups_dev, const BlockDesc *blocks_dev, int n_blocks,
                              size_t smem_bytes, uint32_t seed, uint64_t sweep0, int n_sweeps,
@@ -124,10 +137,22 @@ cudaError_t prepare_scan_kernel(int L, size_t smem_bytes);
 cudaError_t launch_sweeps_scan(int L, const GroupDev *groups_dev, const BlockDesc *blocks_dev,
                                int n_blocks, size_t smem_bytes, uint32_t seed, uint64_t sweep0,
                                int n_sweeps, int64_t ts_pos, bool record, cudaStream_t st);
-// Sweeps of groups with couplings per bond (bonds.cu): blocks of one warp,
-// one thread per walker, BlockDesc.nw <= 32 walkers (P = 1); one launch per
-// row length L, on blocks that all belong to groups of that L.
-cudaError_t launch_sweeps_bonds(int L, const GroupDev *groups_dev, const BlockDesc *blocks_dev,
+// Site-per-lane launch (rows.cu), 3 <= L <= 64, with or without couplings per
+// bond: a walker's row is cut into seg segments of `lanes` consecutive sites,
+// one site per lane, and a block (one warp) serves per_warp = 32 / lanes
+// walkers.  One launch per group; seg = 0: not supported.
+struct RowShape {
+    int seg, lanes, per_warp;
+};
+RowShape rows_shape(int L);
+// Words per row of a lattice kept walker by walker.
+int rows_lattice_words(int L);
+cudaError_t launch_sweeps_rows(const GroupDev &g, uint32_t seed, uint64_t sweep0, int n_sweeps,
+                               int64_t ts_pos, bool record, cudaStream_t st);
+// Sweeps of groups with couplings per bond that the site-per-lane kernel does
+// not cover (bonds.cu, L = 2): blocks of one warp, one thread per walker,
+// BlockDesc.nw <= 32 walkers (P = 1).
+cudaError_t launch_sweeps_bonds(const GroupDev *groups_dev, const BlockDesc *blocks_dev,
                                 int n_blocks, uint32_t seed, uint64_t sweep0, int n_sweeps,
                                 int64_t ts_pos, bool record, cudaStream_t st);
 // Bytes of one walker's lattice (padded rows), of a shared-memory tile, and of

@@ -51,11 +51,10 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKeys &k)
 {
 #pragma unroll
     for (int round = 0; round < 10; ++round) {
-        const uint32_t lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = make_uint4(hi1 ^ c.y ^ k.k0[round], lo1, hi0 ^ c.w ^ k.k1[round], lo0);
+        // one 32 x 32 -> 64 multiply gives both halves
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c.x, p1 = (uint64_t)0xCD9E8D57u * c.z;
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k.k0[round], (uint32_t)p1,
+                       (uint32_t)(p0 >> 32) ^ c.w ^ k.k1[round], (uint32_t)p0);
     }
     return c;
 }

@@ -26,11 +26,12 @@ thread_local std::string g_last_error = "no error";
 
 struct Group {
     muca_group spec{};
-    int L = 0, V = 0, W = 0, Wpad = 0, Lw = 0, e_min = 0, e_max = 0, nE = 0;
+    int L = 0, V = 0, W = 0, Wpad = 0, Lw = 0, rw = 0, e_min = 0, e_max = 0, nE = 0;
     double T = 0, beta = 0;
     uint32_t walker0 = 0;
     // device
-    uint32_t *spins = nullptr;  // [L * L][Lw][Wpad] packed words
+    uint32_t *spins = nullptr;  // packed words, walker-minor or walker by walker (by_walker)
+    bool by_walker = false;     // the layout of spins (muca_internal.h); fixed at init
     int32_t *tal = nullptr;
     unsigned long long *hist = nullptr;
     uint32_t *thr = nullptr;    // table allocation, table_rows(nE) x kRow
@@ -65,6 +66,9 @@ struct Group {
     int P = 1;     // lanes per walker
 };
 
+// Streams for the launches of one sweep call that run side by side.
+constexpr size_t kRangeStreams = 32;
+
 struct GraphKey {
     int n_iters, sweeps;
     uint64_t sweep0;
@@ -98,10 +102,12 @@ struct muca_ctx {
         size_t smem;
     };
     std::vector<ScanRange> scan_ranges;
-    // the disordered model's blocks (kind 5), sorted by L: one launch per L
-    std::vector<ScanRange> bond_ranges;
-    std::vector<cudaStream_t> scan_streams;
-    std::vector<cudaEvent_t> scan_events;
+    // the groups of the site-per-lane kind, one launch each, largest L first
+    std::vector<int> rows_groups;
+    // streams of the row-scan ranges' and the site-per-lane groups' launches, in
+    // this order, taken in turn when there are more launches than streams
+    std::vector<cudaStream_t> range_streams;
+    std::vector<cudaEvent_t> range_events;
 };
 
 namespace {
@@ -178,7 +184,10 @@ void parallel_rows(int n, F f)
 void build_bonds_table(Group &g)
 {
     const int nj = 24 * g.jmax + 1, off = 12 * g.jmax;
-    uint32_t *T = g.h_thrJ;
+    const size_t pad = (size_t)kPad * 3 * nj;
+    std::memset(g.h_thrJ, 0, pad * sizeof(uint32_t));
+    std::memset(g.h_thrJ + pad + (size_t)g.nE * 3 * nj, 0, pad * sizeof(uint32_t));
+    uint32_t *T = g.h_thrJ + pad;
     parallel_rows(g.nE, [&g, T, nj, off](int b, int e_end) {
         for (int e = b; e < e_end; ++e)
             for (int d = -1; d <= 1; ++d)
@@ -187,7 +196,10 @@ void build_bonds_table(Group &g)
     });
 }
 
-size_t bonds_table_words(const Group &g) { return (size_t)g.nE * 3 * (24 * g.jmax + 1); }
+size_t bonds_table_words(const Group &g)
+{
+    return ((size_t)g.nE + 2 * kPad) * 3 * (24 * g.jmax + 1);
+}
 
 // The table a group's sweeps read: its bytes, host copy and device copy.
 size_t table_bytes(const Group &g)
@@ -208,7 +220,7 @@ void build_packed(Group &g)
     }
     uint32_t *T = g.h_thr;
     std::memset(T, 0, table_rows(g.nE) * kRow * sizeof(uint32_t));
-    uint32_t *E0 = T + (size_t)kGuard * kRow;
+    uint32_t *E0 = T + (size_t)(kPad + kGuard) * kRow;
     uint32_t d0[kBlk];
     // d = 0 keeps E_Delta: the same entries in every row (taken in the window)
     for (int k = 0; k < kBlk; ++k) d0[k] = thr_entry(g, g.win_lo, 0, 2 * k - 12);
@@ -235,7 +247,7 @@ int pack_logical(muca_ctx *ctx, Group &g, const uint32_t *lg)
                             "set_table: d = 0 entries must not depend on E_Delta (row %d)", e);
     uint32_t *T = g.h_thr;
     std::memset(T, 0, table_rows(g.nE) * kRow * sizeof(uint32_t));
-    uint32_t *E0 = T + (size_t)kGuard * kRow;
+    uint32_t *E0 = T + (size_t)(kPad + kGuard) * kRow;
     for (int e = 0; e < g.nE; ++e) {
         const uint32_t *r = lg + (size_t)e * 3 * MUCA_NK;
         uint32_t *row = E0 + (size_t)e * kRow;
@@ -344,15 +356,51 @@ GroupDev dev_of(const Group &g)
     d.nE = g.nE;
     d.walker0 = g.walker0;
     d.spins = g.spins;
+    d.wstr = g.by_walker ? 1 : g.Wpad;
+    d.cstr = g.by_walker ? (int64_t)g.L * g.L * g.rw : 1;
+    d.rw = g.rw;
     d.tal = g.tal;
     d.hist = g.hist;
-    d.thrE = g.thr ? g.thr + (size_t)kGuard * kRow : nullptr;
+    d.thrE = g.thr ? g.thr + (size_t)(kPad + kGuard) * kRow : nullptr;
     d.ts = g.ts;
     d.J = g.jmax ? g.d_J : nullptr;
     d.jmax = g.jmax;
-    d.thrJ = g.jmax ? g.thrJ : nullptr;
+    d.thrJ = g.jmax ? g.thrJ + (size_t)kPad * 3 * (24 * g.jmax + 1) : nullptr;
     d.J6 = g.jmax ? g.d_J6 : nullptr;
     return d;
+}
+
+// Words of the group's spins on the device.
+inline size_t lattice_words(const Group &g) { return (size_t)g.L * g.L * g.rw * g.Wpad; }
+
+// Index of packed word j of row `row` of walker w in the group's spins.
+inline size_t word_at(const Group &g, int row, int j, int w)
+{
+    const size_t v = (size_t)row * g.rw + j;
+    return g.by_walker ? (size_t)w * ((size_t)g.L * g.L * g.rw) + v : v * g.Wpad + w;
+}
+
+// The spins of a group in the walker-minor order of the checkpoint file from
+// the group's own order, and back.
+std::vector<uint32_t> to_file_order(const Group &g, const std::vector<uint32_t> &own)
+{
+    if (!g.by_walker) return own;
+    std::vector<uint32_t> out((size_t)g.L * g.L * g.Lw * g.Wpad);
+    for (int w = 0; w < g.Wpad; ++w)
+        for (int row = 0; row < g.L * g.L; ++row)
+            for (int j = 0; j < g.Lw; ++j)
+                out[((size_t)row * g.Lw + j) * g.Wpad + w] = own[word_at(g, row, j, w)];
+    return out;
+}
+std::vector<uint32_t> from_file_order(const Group &g, const std::vector<uint32_t> &file)
+{
+    if (!g.by_walker) return file;
+    std::vector<uint32_t> own(lattice_words(g), 0u);
+    for (int w = 0; w < g.Wpad; ++w)
+        for (int row = 0; row < g.L * g.L; ++row)
+            for (int j = 0; j < g.Lw; ++j)
+                own[word_at(g, row, j, w)] = file[((size_t)row * g.Lw + j) * g.Wpad + w];
+    return own;
 }
 
 int upload_groups(muca_ctx *ctx)
@@ -363,9 +411,16 @@ int upload_groups(muca_ctx *ctx)
     return MUCA_OK;
 }
 
-// Kernel kind of a group's configuration.
+// Whether the site-per-lane kernel sweeps the group.
+bool on_rows(const Group &g)
+{
+    return rows_shape(g.L).seg > 0 && (g.jmax > 0 || g.residency == MUCA_RES_ROWS);
+}
+
+// Kernel kind of a group's block list (-1: none, the site-per-lane kernel).
 int kind_of(const Group &g)
 {
+    if (on_rows(g)) return -1;
     if (g.jmax) return 5;
     if (g.residency == MUCA_RES_SCAN) return 4;
     if (g.residency == MUCA_RES_SPLIT) return g.L > kWsNarrowMaxL ? 3 : 2;
@@ -397,11 +452,16 @@ int bonds_walkers_per_warp(int W)
 
 int build_blocks(muca_ctx *ctx)
 {
+    ctx->rows_groups.clear();
     std::vector<BlockDesc> b[kKinds];
     size_t sm[kKinds] = {};
     for (size_t gi = 0; gi < ctx->g.size(); ++gi) {
         const Group &g = ctx->g[gi];
         const int k = kind_of(g);
+        if (k < 0) {
+            ctx->rows_groups.push_back((int)gi);
+            continue;
+        }
         const size_t need = k == 0   ? stage_bytes_for(g.wpb)
                             : k == 1 ? smem_bytes_for(g.L, g.wpb) + stage_bytes_for(g.wpb)
                             : k == 4 ? scan_bytes_for(g.L)
@@ -412,6 +472,9 @@ int build_blocks(muca_ctx *ctx)
         for (int w0 = 0; w0 < g.W; w0 += wpb)
             b[k].push_back(BlockDesc{(int)gi, w0, std::min(wpb, g.W - w0), wpb, P});
     }
+    // the site-per-lane launches: the longest (most rows per walker) first
+    std::stable_sort(ctx->rows_groups.begin(), ctx->rows_groups.end(),
+                     [&](int x, int y) { return ctx->g[x].L > ctx->g[y].L; });
     // Longest blocks first: when a launch needs more than one wave of blocks,
     // the blocks of the largest lattices (work per sweep: walkers x sites)
     // start first instead of forming the tail.  Row-scan blocks are grouped
@@ -419,16 +482,9 @@ int build_blocks(muca_ctx *ctx)
     for (int k = 0; k < kKinds; ++k)
         std::stable_sort(b[k].begin(), b[k].end(), [&](const BlockDesc &x, const BlockDesc &y) {
             const int lx = ctx->g[x.group].L, ly = ctx->g[y.group].L;
-            if ((k == 4 || k == 5) && lx != ly) return lx > ly;
+            if (k == 4 && lx != ly) return lx > ly;
             return (int64_t)x.nw * ctx->g[x.group].V > (int64_t)y.nw * ctx->g[y.group].V;
         });
-    ctx->bond_ranges.clear();
-    for (int i = 0; i < (int)b[5].size(); ++i) {
-        const int L = ctx->g[b[5][i].group].L;
-        if (ctx->bond_ranges.empty() || ctx->bond_ranges.back().L != L)
-            ctx->bond_ranges.push_back({L, i, 0, 0});
-        ++ctx->bond_ranges.back().count;
-    }
     ctx->scan_ranges.clear();
     for (int i = 0; i < (int)b[4].size(); ++i) {
         const int L = ctx->g[b[4][i].group].L;
@@ -442,13 +498,14 @@ int build_blocks(muca_ctx *ctx)
                         rg.smem);
         CK(prepare_scan_kernel(rg.L, rg.smem));
     }
-    while (ctx->scan_streams.size() < ctx->scan_ranges.size()) {
+    while (ctx->range_streams.size() <
+           std::min(ctx->scan_ranges.size() + ctx->rows_groups.size(), kRangeStreams)) {
         cudaStream_t s = nullptr;
         cudaEvent_t e = nullptr;
         CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-        ctx->scan_streams.push_back(s);
+        ctx->range_streams.push_back(s);
         CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        ctx->scan_events.push_back(e);
+        ctx->range_events.push_back(e);
     }
     for (int k = 0; k < kKinds; ++k) {
         if (sm[k] > 0 && (int64_t)sm[k] + 1024 > (int64_t)max_smem_per_block())
@@ -476,21 +533,29 @@ int build_blocks(muca_ctx *ctx)
 // in use, otherwise forked over per-launch streams and joined.
 int launch_all(muca_ctx *ctx, int n_sweeps, bool record, cudaStream_t st)
 {
-    int used = (int)ctx->scan_ranges.size();
+    const size_t n_scan = ctx->scan_ranges.size(), n_range = n_scan + ctx->rows_groups.size();
+    int used = (int)n_range;
     for (int k = 0; k < 4; ++k) used += ctx->n_blocks[k] > 0;
     used += ctx->n_blocks[5] > 0;
     const bool fork = used > 1;
+    const size_t n_streams = ctx->range_streams.size();
     if (fork) CK(cudaEventRecord(ctx->ev_fork, st));
-    for (size_t i = 0; i < ctx->scan_ranges.size(); ++i) {
-        const auto &rg = ctx->scan_ranges[i];
-        cudaStream_t s = fork ? ctx->scan_streams[i] : st;
-        if (fork) CK(cudaStreamWaitEvent(s, ctx->ev_fork, 0));
-        CK(launch_sweeps_scan(rg.L, ctx->d_groups, ctx->d_blocks[4] + rg.first, rg.count, rg.smem,
-                              ctx->seed, ctx->sweep, n_sweeps, ctx->ts_len, record, s));
-        if (fork) {
-            CK(cudaEventRecord(ctx->scan_events[i], s));
-            CK(cudaStreamWaitEvent(st, ctx->scan_events[i], 0));
+    for (size_t i = 0; i < n_range; ++i) {
+        cudaStream_t s = fork ? ctx->range_streams[i % n_streams] : st;
+        if (fork && i < n_streams) CK(cudaStreamWaitEvent(s, ctx->ev_fork, 0));
+        if (i < n_scan) {
+            const auto &rg = ctx->scan_ranges[i];
+            CK(launch_sweeps_scan(rg.L, ctx->d_groups, ctx->d_blocks[4] + rg.first, rg.count,
+                                  rg.smem, ctx->seed, ctx->sweep, n_sweeps, ctx->ts_len, record,
+                                  s));
+        } else {
+            CK(launch_sweeps_rows(dev_of(ctx->g[ctx->rows_groups[i - n_scan]]), ctx->seed,
+                                  ctx->sweep, n_sweeps, ctx->ts_len, record, s));
         }
+    }
+    for (size_t i = 0; fork && i < std::min(n_range, n_streams); ++i) {
+        CK(cudaEventRecord(ctx->range_events[i], ctx->range_streams[i]));
+        CK(cudaStreamWaitEvent(st, ctx->range_events[i], 0));
     }
     for (int k = 0; k < 4; ++k) {
         if (ctx->n_blocks[k] == 0) continue;
@@ -510,9 +575,8 @@ int launch_all(muca_ctx *ctx, int n_sweeps, bool record, cudaStream_t st)
     if (ctx->n_blocks[5] > 0) {
         cudaStream_t s = fork ? ctx->side[5] : st;
         if (fork) CK(cudaStreamWaitEvent(s, ctx->ev_fork, 0));
-        for (const auto &rg : ctx->bond_ranges)
-            CK(launch_sweeps_bonds(rg.L, ctx->d_groups, ctx->d_blocks[5] + rg.first, rg.count,
-                                   ctx->seed, ctx->sweep, n_sweeps, ctx->ts_len, record, s));
+        CK(launch_sweeps_bonds(ctx->d_groups, ctx->d_blocks[5], ctx->n_blocks[5], ctx->seed,
+                               ctx->sweep, n_sweeps, ctx->ts_len, record, s));
         if (fork) {
             CK(cudaEventRecord(ctx->ev_join[5], s));
             CK(cudaStreamWaitEvent(st, ctx->ev_join[5], 0));
@@ -625,6 +689,12 @@ std::map<std::tuple<int, int, int, int, int>, Cand> g_tune_cache;
 static int tune_group(muca_ctx *ctx, size_t gi, int residency, int wpb, int P)
 {
     Group &g = ctx->g[gi];
+    if (g.by_walker) {
+        g.residency = MUCA_RES_ROWS;
+        g.wpb = rows_shape(g.L).per_warp;
+        g.P = rows_shape(g.L).lanes;
+        return MUCA_OK;
+    }
     const int smem_max = max_smem_per_block();
     std::vector<Cand> cands = candidates(g, residency, wpb, P, smem_max);
     if (cands.empty())
@@ -650,7 +720,7 @@ static int tune_group(muca_ctx *ctx, size_t gi, int residency, int wpb, int P)
         }
     }
     // scratch copy of the state
-    const size_t sb = (size_t)g.L * g.L * g.Lw * g.Wpad * sizeof(uint32_t), tb = (size_t)3 * g.Wpad * sizeof(int32_t),
+    const size_t sb = lattice_words(g) * sizeof(uint32_t), tb = (size_t)3 * g.Wpad * sizeof(int32_t),
                  hb = (size_t)g.nE * sizeof(unsigned long long);
     uint32_t *s0 = nullptr;
     int32_t *t0 = nullptr;
@@ -761,7 +831,7 @@ static int tune_batch(muca_ctx *ctx)
     for (size_t i = 0; i < n && rc == MUCA_OK; ++i) {
         const Group &g = ctx->g[i];
         Backup &b = bk[i];
-        b.sb = (size_t)g.L * g.L * g.Lw * g.Wpad * sizeof(uint32_t);
+        b.sb = lattice_words(g) * sizeof(uint32_t);
         b.tb = (size_t)3 * g.Wpad * sizeof(int32_t);
         b.hb = (size_t)g.nE * sizeof(unsigned long long);
         if (cudaMalloc(&b.s, b.sb) != cudaSuccess || cudaMalloc(&b.t, b.tb) != cudaSuccess ||
@@ -874,8 +944,8 @@ void muca_destroy(muca_ctx *ctx)
         if (ctx->ev_join[k]) cudaEventDestroy(ctx->ev_join[k]);
         cudaFree(ctx->d_blocks[k]);
     }
-    for (auto s : ctx->scan_streams) cudaStreamDestroy(s);
-    for (auto e : ctx->scan_events) cudaEventDestroy(e);
+    for (auto s : ctx->range_streams) cudaStreamDestroy(s);
+    for (auto e : ctx->range_events) cudaEventDestroy(e);
     if (ctx->cap) cudaStreamDestroy(ctx->cap);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     delete ctx;
@@ -973,11 +1043,21 @@ int muca_init(const muca_group *groups, int n_groups, const muca_options *opt, v
             g.T = groups[i].T;
             g.beta = 1.0 / g.T;
             g.walker0 = w0 + (uint32_t)lo;
+            g.by_walker = opt->residency == MUCA_RES_AUTO && opt->walkers_per_block == 0 &&
+                          opt->lanes_per_walker == 0 && rows_shape(g.L).seg > 0;
             w0 += (uint32_t)tot;
             g.lnW.assign(g.nE, 0.0);
             g.acc.assign((size_t)std::max(g.nE - 1, 1), 0.0);
-            const size_t sbytes = (size_t)g.L * g.L * g.Lw * g.Wpad * sizeof(uint32_t);
-            CKI(cudaMalloc(&g.spins, sbytes));
+            g.rw = g.by_walker ? rows_lattice_words(g.L) : g.Lw;
+            if (g.by_walker && cudaMalloc(&g.spins, lattice_words(g) * sizeof(uint32_t)) != cudaSuccess) {
+                // no room for padded rows: the walker-minor layout and its kernels
+                (void)cudaGetLastError();
+                g.spins = nullptr;
+                g.by_walker = false;
+                g.rw = g.Lw;
+            }
+            const size_t sbytes = lattice_words(g) * sizeof(uint32_t);
+            if (!g.spins) CKI(cudaMalloc(&g.spins, sbytes));
             CKI(cudaMemsetAsync(g.spins, 0, sbytes, ctx->stream));
             CKI(cudaMalloc(&g.tal, (size_t)3 * g.Wpad * sizeof(int32_t)));
             CKI(cudaMemsetAsync(g.tal, 0, (size_t)3 * g.Wpad * sizeof(int32_t), ctx->stream));
@@ -1560,15 +1640,14 @@ int muca_get_state(muca_ctx *ctx, int group, int8_t *spins, int32_t *tallies)
     if (rc) return rc;
     Group &g = ctx->g[group];
     if (spins) {
-        const size_t nwords = (size_t)g.L * g.L * g.Lw;
-        std::vector<uint32_t> dev(nwords * g.Wpad);
+        std::vector<uint32_t> dev(lattice_words(g));
         CK(cudaMemcpyAsync(dev.data(), g.spins, dev.size() * sizeof(uint32_t),
                            cudaMemcpyDeviceToHost, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
         for (int w = 0; w < g.W; ++w)
             for (int row = 0; row < g.L * g.L; ++row)
                 for (int x = 0; x < g.L; ++x) {
-                    const uint32_t word = dev[((size_t)row * g.Lw + (x >> 2)) * g.Wpad + w];
+                    const uint32_t word = dev[word_at(g, row, x >> 2, w)];
                     spins[(size_t)w * g.V + (size_t)row * g.L + x] =
                         (int8_t)(uint8_t)(word >> (8 * (x & 3)));
                 }
@@ -1590,8 +1669,7 @@ int muca_set_state(muca_ctx *ctx, int group, const int8_t *spins)
     if (rc) return rc;
     if (!spins) return fail(ctx, MUCA_ERR_INVALID_ARG, "spins is NULL");
     Group &g = ctx->g[group];
-    const size_t nwords = (size_t)g.L * g.L * g.Lw;
-    std::vector<uint32_t> dev(nwords * g.Wpad, 0u);
+    std::vector<uint32_t> dev(lattice_words(g), 0u);
     for (int w = 0; w < g.W; ++w)
         for (int row = 0; row < g.L * g.L; ++row)
             for (int x = 0; x < g.L; ++x) {
@@ -1599,7 +1677,7 @@ int muca_set_state(muca_ctx *ctx, int group, const int8_t *spins)
                 if (s < -1 || s > 1)
                     return fail(ctx, MUCA_ERR_INVALID_ARG, "walker %d site %d: spin %d", w,
                                 row * g.L + x, s);
-                dev[((size_t)row * g.Lw + (x >> 2)) * g.Wpad + w] |=
+                dev[word_at(g, row, x >> 2, w)] |=
                     (uint32_t)(uint8_t)s << (8 * (x & 3));
             }
     std::vector<int32_t> old((size_t)3 * g.Wpad);
@@ -1644,9 +1722,12 @@ int muca_get_config(muca_ctx *ctx, int group, int32_t *residency, int32_t *walke
     int rc = check_group_index(ctx, group);
     if (rc) return rc;
     const Group &g = ctx->g[group];
+    const RowShape rows = rows_shape(g.L);
+    const bool lane = g.jmax && on_rows(g);  // couplings on the site-per-lane kernel
     if (residency) *residency = g.jmax ? MUCA_RES_BONDS : g.residency;
-    if (walkers_per_block) *walkers_per_block = g.jmax ? bonds_walkers_per_warp(g.W) : g.wpb;
-    if (lanes_per_walker) *lanes_per_walker = g.jmax ? 1 : g.P;
+    if (walkers_per_block)
+        *walkers_per_block = lane ? rows.per_warp : g.jmax ? bonds_walkers_per_warp(g.W) : g.wpb;
+    if (lanes_per_walker) *lanes_per_walker = lane ? rows.lanes : g.jmax ? 1 : g.P;
     return MUCA_OK;
 }
 
@@ -1700,7 +1781,7 @@ int muca_checkpoint(muca_ctx *ctx, const char *path)
         if (!ok) break;
         std::vector<unsigned long long> h(g.nE);
         std::vector<int32_t> t((size_t)3 * g.Wpad);
-        std::vector<uint32_t> s((size_t)g.L * g.L * g.Lw * g.Wpad);
+        std::vector<uint32_t> s(lattice_words(g));
         if (cudaMemcpy(h.data(), g.hist, h.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess ||
             cudaMemcpy(t.data(), g.tal, t.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
             cudaMemcpy(s.data(), g.spins, s.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess) {
@@ -1710,6 +1791,7 @@ int muca_checkpoint(muca_ctx *ctx, const char *path)
         ok = ok && std::fwrite(g.lnW.data(), 8, g.nE, f) == (size_t)g.nE;
         ok = ok && std::fwrite(g.acc.data(), 8, g.acc.size(), f) == g.acc.size();
         ok = ok && std::fwrite(h.data(), 8, h.size(), f) == h.size();
+        s = to_file_order(g, s);
         ok = ok && std::fwrite(t.data(), 4, t.size(), f) == t.size();
         ok = ok && std::fwrite(s.data(), 4, s.size(), f) == s.size();
     }
@@ -1806,6 +1888,7 @@ int muca_restore(muca_ctx *ctx, const char *path)
             std::fclose(f);
             return fail(ctx, MUCA_ERR_IO, "restore: %s is truncated", path);
         }
+        s = from_file_order(g, s);
         g.lnW = lnW;
         g.acc = acc;
         g.recursion = recs[gi];

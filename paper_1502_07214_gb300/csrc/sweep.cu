@@ -1249,7 +1249,7 @@ __global__ void init_spins_kernel(GroupDev g, uint32_t seed)
             const int v = (int)(((uint64_t)rq * 3u) >> 32) - 1;
             word |= (uint32_t)(v & 0xFF) << (8 * q);
         }
-        g.spins[wd * g.Wpad + w] = word;
+        g.spins[((int64_t)row * g.rw + j) * g.wstr + w * g.cstr] = word;
     }
 }
 
@@ -1261,9 +1261,9 @@ __global__ void energies_kernel(GroupDev g, int mode, int *err)
 {
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
     if (w >= g.W) return;
-    const int L = g.L, Lw = g.Lw;
-    uint32_t *lat = g.spins + w;
-    const ptrdiff_t st = g.Wpad;
+    const int L = g.L, rw = g.rw;
+    uint32_t *lat = g.spins + (ptrdiff_t)w * g.cstr;
+    const ptrdiff_t st = g.wstr;
     int ej = 0, ed = 0, m = 0;
     for (int z = 0; z < L; ++z) {
         const int zp = (z + 1 == L) ? 0 : z + 1;
@@ -1271,13 +1271,13 @@ __global__ void energies_kernel(GroupDev g, int mode, int *err)
             const int yp = (y + 1 == L) ? 0 : y + 1;
             for (int x = 0; x < L; ++x) {
                 const int xp = (x + 1 == L) ? 0 : x + 1;
-                const int s = *site_ptr(lat, st, Lw, z * L + y, x);
+                const int s = *site_ptr(lat, st, rw, z * L + y, x);
                 const int i = x + L * (y + L * z);
                 const int jx = g.J ? g.J[3 * i + 0] : 1, jy = g.J ? g.J[3 * i + 1] : 1,
                           jz = g.J ? g.J[3 * i + 2] : 1;
-                ej -= s * (jx * *site_ptr(lat, st, Lw, z * L + y, xp) +
-                           jy * *site_ptr(lat, st, Lw, z * L + yp, x) +
-                           jz * *site_ptr(lat, st, Lw, zp * L + y, x));
+                ej -= s * (jx * *site_ptr(lat, st, rw, z * L + y, xp) +
+                           jy * *site_ptr(lat, st, rw, z * L + yp, x) +
+                           jz * *site_ptr(lat, st, rw, zp * L + y, x));
                 ed += s * s;
                 m += s;
             }

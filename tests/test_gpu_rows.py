@@ -1,0 +1,108 @@
+"""The site-per-lane sweep kernel (the choice of MUCA_RES_AUTO) against the
+oracle, bit for bit: every way a row is laid out on a warp (one segment, rows
+that are no multiple of 4, the last length of each shared-memory row width,
+three and four segments with full and ragged last ones), the hot regime in
+which a row takes many passes, narrow windows, and checkpoints between its
+lattice layout and the walker-minor one."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1502_07214_gb300 import workloads as wl
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+
+def muca():
+    from paper_1502_07214_gb300 import muca as m
+
+    return m
+
+
+def run_against_oracle(L, T, W, lnW, n, bonds=None, e_min=0, e_max=None, spins0=None):
+    V = L ** 3
+    e_max = V if e_max is None else e_max
+    c = muca().Context([{"L": L, "T": T, "n_walkers": W, "e_min": e_min, "e_max": e_max}], seed=L)
+    if spins0 is not None:
+        c.set_state(0, spins0)
+    if bonds is not None:
+        c.set_bonds(0, bonds)
+    assert c.get_config(0)[0] == (muca().RES_ROWS if bonds is None else muca().RES_BONDS)
+    c.set_lnW(0, lnW)
+    c.reserve_timeseries(n)
+    c.sweep_iter(n, record=True)
+    spins, tal = c.get_state(0)
+    ts, H = c.get_timeseries(0), c.get_hist(0)
+    c.check_tallies()
+    c.close()
+    jmax = None if bonds is None else int(np.abs(bonds).max())
+    thr = (oracle.build_table(L, T, e_min, e_max, lnW) if bonds is None else
+           oracle.build_table_bonds(L, T, jmax, e_min, e_max, lnW))
+    for w in range(W):
+        sp = oracle.init_spins(L, L, w) if spins0 is None else spins0[w].copy()
+        if bonds is None:
+            t = oracle.energies(L, sp).astype(np.int32)
+            ref = oracle.sweeps(L, e_min, e_max, thr, L, w, 0, n, sp, t, record=True)
+        else:
+            t = oracle.energies_bonds(L, sp, bonds).astype(np.int32)
+            ref = oracle.sweeps_bonds(L, bonds, jmax, e_min, e_max, thr, L, w, 0, n, sp, t,
+                                      record=True)
+        assert np.array_equal(spins[w], sp) and np.array_equal(tal[w], t), w
+        assert np.array_equal(ts[:, :, w], ref), w
+    assert np.array_equal(H, np.bincount(ts[:, 1, :].ravel() - e_min,
+                                         minlength=len(H)).astype(np.uint64))
+
+
+# (L, walkers): one walker more than whole warps where several share one
+@pytest.mark.parametrize("L,W", [(3, 21), (4, 17), (5, 13), (8, 9), (11, 5), (12, 7), (13, 5),
+                                 (16, 5), (17, 3), (22, 3), (31, 2), (32, 3), (33, 5), (48, 5),
+                                 (49, 3), (61, 3), (64, 3)])
+def test_every_row_layout_under_rough_transition_weights(L, W):
+    """Weights with the transition's slope and a roughness of 0.5 per bin from
+    the random start: some ten accepted moves per row, whose order matters."""
+    T = 1.0
+    lnW = -2.944 / T * np.arange(L ** 3 + 1) + wl.random_lnW(L ** 3 + 1, L, scale=0.5)
+    run_against_oracle(L, T, W, lnW, 3 if L <= 33 else 2)
+
+
+@pytest.mark.parametrize("L,W,jj", [(3, 12, (1, 3)), (7, 6, (-1, 1)), (12, 5, (2, 8)),
+                                    (18, 3, (5, 3)), (32, 2, (0, 2)), (36, 3, (-3, 1))])
+def test_couplings_in_every_row_layout(L, W, jj):
+    lnW = -1.5 * np.arange(L ** 3 + 1) + wl.random_lnW(L ** 3 + 1, L, scale=0.5)
+    run_against_oracle(L, 3.0, W, lnW, 2, bonds=wl.random_bonds(L, jj[0], jj[1], seed=L))
+
+
+@pytest.mark.parametrize("e_min,e_max", [(256, 256), (250, 262), (0, 300), (200, 512)])
+def test_narrow_windows(e_min, e_max):
+    L, W = 8, 6
+    rng = np.random.default_rng(4)
+    spins = np.zeros((W, L ** 3), dtype=np.int8)
+    for w in range(W):
+        at = rng.permutation(L ** 3)[:256]
+        spins[w, at] = rng.choice(np.array([-1, 1], dtype=np.int8), 256)
+    run_against_oracle(L, 1.4182, W, wl.random_lnW(e_max - e_min + 1, 3), 20, e_min=e_min,
+                       e_max=e_max, spins0=spins)
+
+
+@pytest.mark.parametrize("L", [6, 20, 34])
+def test_checkpoints_cross_lattice_layouts(L, tmp_path):
+    """A file written from one layout continues bit-identically in the other."""
+    g = [{"L": L, "T": 1.4182, "n_walkers": 5}]
+    a = muca().Context(g, seed=7)
+    b = muca().Context(g, seed=7, residency=muca().RES_GLOBAL, walkers_per_block=32)
+    assert a.get_config(0)[0] == muca().RES_ROWS and b.get_config(0)[0] == muca().RES_GLOBAL
+    a.sweep_iter(3)
+    pa, pb = str(tmp_path / "a"), str(tmp_path / "b")
+    a.checkpoint(pa)
+    b.restore(pa)
+    b.sweep_iter(2)
+    b.checkpoint(pb)
+    a.sweep_iter(2)
+    want = a.get_state(0)
+    a.restore(pb)
+    for c in (a, b):
+        got = c.get_state(0)
+        assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+        c.close()
