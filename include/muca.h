@@ -323,7 +323,8 @@ int muca_reweight(const int32_t *e_j, const int32_t *e_d, const int32_t *m, int6
  * reserve all device memory up front, real-time loops that cannot afford an
  * allocator's synchronisation, bindings without a device allocator.
  * Arguments, layouts, results and errors are those of muca_reweight.  Its
- * working memory is a fixed 4 MiB array in the library's device memory,
+ * working memory is a fixed array in the library's device memory (4 MiB for the
+ * sums and 8 MiB for the coefficients of the FP64 grid),
  * present on every GPU that loads the library until the process exits; this
  * covers n_e <= 32769 (an L = 32 lattice) with n_grid <= 4096 in either
  * precision, and larger problems fail with MUCA_ERR_INVALID_ARG.  The first

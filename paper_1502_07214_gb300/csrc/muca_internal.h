@@ -181,6 +181,11 @@ int reweight_on_scratch(const int32_t *e_j, const int32_t *e_d, const int32_t *m
                         int32_t row_len, int64_t row_stride, const double *lnW, int32_t e_min,
                         int32_t n_e, double beta, int32_t V, const double *delta_grid,
                         int32_t n_grid, int32_t precision, double *out, cudaStream_t st,
-                        char *scratch, char *records = nullptr, size_t records_bytes = 0);
+                        char *scratch, char *records, size_t records_bytes, char *blocks,
+                        size_t blocks_bytes);
+// blocks / blocks_bytes: a third region, of at least reweight_block_bytes(...)
+// bytes, for the coefficients of FP64 stage B's blocks of bins.
+size_t reweight_block_bytes(double beta, const double *delta_grid, int32_t n_grid, int32_t n_e,
+                            int32_t precision);
 
 }  // namespace muca

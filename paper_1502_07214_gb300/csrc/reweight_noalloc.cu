@@ -34,10 +34,12 @@
 namespace {
 
 // 4 MiB: enough for n_e <= 32769 E_Delta bins (an L = 32 lattice) with
-// n_grid <= 4096 Delta points in either precision.
-constexpr size_t kScratchBytes = size_t(4) << 20;
+// n_grid <= 4096 Delta points in either precision.  Behind them 8 MiB for the
+// coefficients of FP64 stage B's blocks of bins: a problem that fits the first
+// part has at most 37000 bins, and blocks take at most 170 bytes per bin.
+constexpr size_t kScratchBytes = size_t(4) << 20, kBlockBytes = size_t(8) << 20;
 
-static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
+static __device__ __align__(256) unsigned char g_scratch[kScratchBytes + kBlockBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
@@ -99,5 +101,6 @@ extern "C" int muca_reweight_noalloc(const int32_t *e_j, const int32_t *e_d, con
     if (rc != MUCA_OK) return rc;
     return muca::reweight_on_scratch(e_j, e_d, m, n_rows, row_len, row_stride, lnW, e_min, n_e,
                                      beta, V, delta_grid, n_grid, precision, out,
-                                     (cudaStream_t)stream, (char *)scratch);
+                                     (cudaStream_t)stream, (char *)scratch, nullptr, 0,
+                                     (char *)scratch + kScratchBytes, kBlockBytes);
 }

@@ -240,3 +240,27 @@ def test_bucketed_sums_ragged_rows_and_wide_windows():
     b = muca().reweight(dev(ej), dev(ed), dev(m), lnW, 0, 0.5, 64, [0.5, 3.0], 64, no_alloc=True)
     assert np.array_equal(a, b)
     assert np.allclose(a[:, 0], ej.mean(), rtol=1e-12)
+
+
+def test_fp64_blocks_of_bins_every_size():
+    """The FP64 grid stage sums blocks of 1, 8, 16, 32 or 64 bins, by the grid's
+    width: every block size against the oracle, with a last block of one bin,
+    empty blocks, a single field, fields in no order, and weights that move by
+    hundreds within a block (the edges of a real density of states)."""
+    rng = np.random.default_rng(8)
+    n_e, beta = 64 * 9 + 1, 0.8
+    ed = np.concatenate([rng.integers(0, 200, 3000), rng.integers(400, n_e, 3000)])
+    ej = -2 * ed + rng.integers(-40, 41, ed.size)
+    m = np.clip(rng.integers(-n_e, n_e, ed.size), -ed, ed)
+    e = np.arange(n_e)
+    smooth = -beta * 2.0 * e + 0.3 * np.sin(e / 7.0)
+    # ln of a binomial-like density of states: slopes up to ln(n_e), then steps of 150
+    edge = -beta * 2.0 * e - 8.0 * np.sqrt(e * (n_e - e + 1.0)) / 10 + 150.0 * (e % 29 == 0)
+    for lnW in (smooth, edge):
+        for width in (0.0, 0.02, 0.05, 0.1, 0.25, 0.7, 3.0):  # 64, 64, 32, 16, 8, 1, 1 bins
+            grid = 2.0 + width * (rng.random(7) - 0.5) if width else np.array([2.0])
+            if width:
+                grid[:2] = 2.0 - width / 2, 2.0 + width / 2
+            ref = oracle.reweight(ej, ed, m, lnW, 0, beta, n_e - 1, grid)
+            got = muca().reweight(dev(ej), dev(ed), dev(m), lnW, 0, beta, n_e - 1, grid, 64)
+            assert (rel_err(got, ref) <= TOL[64]).all(), (width, rel_err(got, ref).max(axis=0))
