@@ -198,3 +198,27 @@ def test_equal_height_errors():
     with pytest.raises(muca().MucaError) as e:
         muca().equal_height(dev(bad), lnW, 0, beta, int(0.525 * V), dt - 0.05, dt + 0.05)
     assert e.value.code == muca().ERR_WINDOW
+
+
+@pytest.mark.parametrize("scale,jack", [(1.0, 0), (0.5, 2), (0.15, 3), (0.002, 6), (1e-4, 70)])
+def test_peak_blocks_of_bins_every_size(scale, jack):
+    """The bisection sums blocks of bins as large as the interval allows: wide
+    and narrow intervals (single bins to 512), one to several CTAs per data set
+    and more sets than SMs hold clusters of, against the oracle."""
+    L, T = 12, 1.4182
+    beta, V = 1 / T, L ** 3
+    ej, ed, m, lnW, dt = wl.synthetic_series(L=L, T=T, n_walkers=512, n_samples=1400, seed=6)
+    lo, hi = bracket(ej, ed, m, lnW, beta, V, dt, n=31, k_side=3)
+    c = oracle.find_peak(ej, ed, lnW, 0, beta, lo, hi, n_iter=60, n_jack=0)[0, 0]
+    # the interval shrinks about Delta*, but not past the subsets' spread
+    spread = 0.0
+    if jack:
+        sub = oracle.find_peak(ej, ed, lnW, 0, beta, lo, hi, n_iter=60, n_jack=jack)[:, 0]
+        spread = 2.0 * np.abs(sub - c).max()
+    a, b = c - max(scale * (c - lo), spread), c + max(scale * (hi - c), spread)
+    ref = oracle.find_peak(ej, ed, lnW, 0, beta, a, b, n_iter=60, n_jack=jack)
+    got = muca().find_peak(dev(ej), dev(ed), lnW, 0, beta, a, b, n_iter=60, n_jack=jack)
+    assert abs(got[0] - ref[0, 0]) <= 1e-9
+    assert abs(got[2] - ref[0, 1]) <= 1e-10 * abs(ref[0, 1])
+    np.testing.assert_allclose(got[4][:, 0], ref[1:, 0], rtol=0, atol=1e-9)
+    np.testing.assert_allclose(got[4][:, 1], ref[1:, 1], rtol=1e-10)
