@@ -1335,10 +1335,10 @@ int reweight_check_args(const int32_t *e_j, const int32_t *e_d, const int32_t *m
 
 }  // namespace muca
 
-// Device memory pool of the reweighting on the current device, created on
-// first use.  It keeps what it has once held (release threshold: all), so that
+// Device memory pool of the analysis calls (muca_reweight, muca_find_peak,
+// muca_equal_height) on the current device, created on first use.  It keeps what it has once held (release threshold: all), so that
 // repeated calls do not map and unmap their working memory each time.
-static int reweight_pool(cudaMemPool_t *out)
+int muca::scratch_pool(cudaMemPool_t *out)
 {
     static std::mutex mu;
     static cudaMemPool_t pools[64] = {};
@@ -1383,7 +1383,7 @@ extern "C" int muca_reweight(const int32_t *e_j, const int32_t *e_d, const int32
     const size_t bytes = muca::reweight_scratch_bytes(n_e, n_grid, precision);
     const size_t rbytes = muca::reweight_record_bytes(n_e, n_rows * (int64_t)row_len);
     cudaMemPool_t pool = nullptr;
-    rc = reweight_pool(&pool);
+    rc = muca::scratch_pool(&pool);
     if (rc != MUCA_OK) return rc;
     void *scratch = nullptr;
     const size_t bbytes = muca::reweight_block_bytes(beta, delta_grid, n_grid, n_e, precision);
