@@ -102,6 +102,18 @@ __device__ __forceinline__ void st_global_v4(void *a, uint4 v, bool p)
                  "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((int)p)
                  : "memory");
 }
+// A spin of the lattice, read once by this lane: not kept in L1, which holds
+// the thresholds.
+__device__ __forceinline__ int ld_lattice(const char *p)
+{
+    int v;
+    asm volatile("ld.global.L1::no_allocate.s8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void prefetch_l2(const void *p, bool on)
+{
+    asm volatile("{.reg .pred q; setp.ne.s32 q, %1, 0; @q prefetch.global.L2 [%0];}" ::"l"(p), "r"((int)on));
+}
 __device__ __forceinline__ void cp4(void *smem, const void *gmem)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(shared_addr(smem)), "l"(gmem) : "memory");
@@ -116,21 +128,36 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 __device__ __forceinline__ void cp_wait_1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Shared memory of one walker: two buffers of random words, then its planes,
-// rows PITCH bytes apart so that a row's addresses are a register and a
-// constant.  A plane has L + 1 rows: row L repeats row 0, the y + 1 neighbour
-// of the last row.  All L planes of a small lattice are held, else the three
-// that a row reads (z - 1, z, z + 1).
-__host__ __device__ constexpr int rows_slots(int L) { return L <= 12 ? L : 3; }
+// How a walker's rows pass through shared memory, by the number of segments
+// (L <= 32: 1, L <= 48: 3, above: 4).
+//   planes: up to 12 sites all L; one and three segments the three planes that
+//     a row reads (z - 1, z, z + 1); four segments plane z alone, whose finished
+//     rows give way to those of plane z + 1, the z neighbours read from the
+//     lattice a step ahead;
+//   row L of a plane repeats row 0, the y + 1 neighbour of the last row, but for
+//     three segments, where a select takes its place;
+//   random words: two buffers for one segment, so that the next rows' words are
+//     stored as they are drawn; else one, the words waiting in registers.
+// The differences buy room: 48-site rows take 15.5 KB per warp, 14 warps per
+// SM, so that the benchmark's 2048 warps run in one wave (17.4 KB left 72 of
+// them to a second one: 157 -> 116 ms for 60 sweeps of 4096 walkers; with
+// plane z alone, the z neighbours' latency gave 146 ms).
+// Rows are PITCH bytes apart, so a row's addresses are a register and a
+// constant.
+__host__ __device__ constexpr int rows_slots(int L) { return L <= 12 ? L : L <= 48 ? 3 : 1; }
+__host__ __device__ constexpr bool rows_repeat0(int seg) { return seg != 3; }
+__host__ __device__ constexpr int rows_buffers(int seg) { return seg == 1 ? 2 : 1; }
 // Words of a buffer: four rows touch at most L + 1 Philox blocks (rows that
 // start inside a block, L odd, one more than L).
 __host__ __device__ constexpr int rows_random_words(int L) { return 4 * (L + 1); }
 // Words from one walker to the next: 16-byte aligned, and spread over the
-// banks so that the walkers of a warp read a row without conflicts.  The words
-// ahead of a plane's last rows are read, and not used: two rows of slack.
-__host__ __device__ inline int rows_walker_words(int L, int per_warp, int pitch)
+// banks so that the walkers of a warp read a row without conflicts.  With one
+// segment the rows after a plane's last are read, and not used: two rows of
+// slack.
+__host__ __device__ inline int rows_walker_words(int L, int seg, int per_warp, int pitch)
 {
-    const int n = 2 * rows_random_words(L) + (rows_slots(L) * (L + 1) + 2) * (pitch / 4);
+    const int rows = rows_slots(L) * (L + rows_repeat0(seg)) + (seg == 1 ? 2 : 0);
+    const int n = rows_buffers(seg) * rows_random_words(L) + rows * (pitch / 4);
     const int want = per_warp <= 1 ? 0 : per_warp == 2 ? 16 : per_warp <= 4 ? 8 : 4;
     return want ? n + ((want - n) % 32 + 32) % 32 : (n + 3) / 4 * 4;
 }
@@ -156,10 +183,10 @@ struct RowCopy {
                     *reinterpret_cast<const uint32_t *>(sm + i * PITCH + 4 * h);
     }
     // a whole plane, and row 0 once more as row L
-    __device__ __forceinline__ void plane_in(int8_t *sm, int z) const
+    __device__ __forceinline__ void plane_in(int8_t *sm, int z, bool repeat0) const
     {
         in(sm, z, 0, L);
-        in(sm + L * PITCH, z, 0, 1);
+        if (repeat0) in(sm + L * PITCH, z, 0, 1);
     }
 };
 
@@ -169,6 +196,10 @@ struct Site {
     int s, delta, d, step;  // old spin, s' - s, s'^2 - s^2, column step per unit of h
     int h;                  // neighbour sum without the y - 1 neighbour
     uint32_t j;             // couplings to the x and y neighbours
+    // from the row's other lanes: the left site's delta, site 0's, and which
+    // sites' moves have d = +1 and d = -1
+    int dl, d0;
+    unsigned Pm, Mm;
 };
 
 // The sweeps of one warp's walkers w0 .. w0 + nw - 1 (a block).  Lane h of a
@@ -202,22 +233,26 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
         xl_o[q] = xo[q] == 0 ? L - 1 : xo[q] - 1;
         xr_o[q] = xo[q] == L - 1 ? 0 : xo[q] + 1;
     }
-    uint32_t *const mem = smem + slot * rows_walker_words(L, per_warp, PITCH);
-    int8_t *const sp = reinterpret_cast<int8_t *>(mem + 2 * rows_random_words(L));
-    const int pb = (L + 1) * PITCH;  // bytes per plane
+    uint32_t *const mem = smem + slot * rows_walker_words(L, SEG, per_warp, PITCH);
+    int8_t *const sp = reinterpret_cast<int8_t *>(mem + rows_buffers(SEG) * rows_random_words(L));
+    constexpr bool REPEAT0 = rows_repeat0(SEG), TWO = rows_buffers(SEG) == 2;
+    const int pb = (L + REPEAT0) * PITCH;  // bytes per plane
     const bool ring = rows_slots(L) < L;
+    constexpr bool OWN = SEG > 3;  // plane z alone in shared memory
     const RowCopy<PITCH> copy{g.spins + (ptrdiff_t)w * g.cstr, g.wstr, L, g.Lw, g.rw, h};
     // a lattice whose rows lie as in shared memory is copied 16 bytes per lane
     const bool wide = g.wstr == 1 && g.rw * 4 == PITCH;
     char *const lat = reinterpret_cast<char *>(copy.g) + 16 * h;
     const uint32_t sp_a = shared_addr(sp);
     if (used) {
-        if (ring) {
-            copy.plane_in(sp, L - 1);
-            copy.plane_in(sp + pb, 0);
-            copy.plane_in(sp + 2 * pb, 1);
+        if (OWN) {
+            copy.plane_in(sp, 0, REPEAT0);
+        } else if (ring) {
+            copy.plane_in(sp, L - 1, REPEAT0);
+            copy.plane_in(sp + pb, 0, REPEAT0);
+            copy.plane_in(sp + 2 * pb, 1, REPEAT0);
         } else {
-            for (int z = 0; z < L; ++z) copy.plane_in(sp + z * pb, z);
+            for (int z = 0; z < L; ++z) copy.plane_in(sp + z * pb, z, REPEAT0);
         }
     }
     cp_commit();
@@ -226,7 +261,8 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
     const int trow = BONDS ? 3 * nj : kRow;
     const uint32_t *__restrict__ thr = (BONDS ? g.thrJ : g.thrE) - (ptrdiff_t)kPad * trow +
                                        (BONDS ? nj + 12 * g.jmax : 19);
-    const unsigned lower = ((1u << lane) - 1u) & ((A == 32 ? ~0u : ((1u << A) - 1u)) << sbase);
+    const unsigned lanes = (A == 32 ? ~0u : ((1u << A) - 1u)) << sbase;  // the walker's
+    const unsigned lower = ((1u << lane) - 1u) & lanes;
     const int last_lane = sbase + (L - 1) - (SEG - 1) * A;  // holds site L - 1
     const unsigned bitL = h > 0 ? 1u << (lane - 1) : 0u;
     const unsigned bit0 = SEG == 1 && lane == last_lane ? 1u << sbase : 0u;
@@ -236,19 +272,27 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
     int eo = (g.tal[g.Wpad + w] - g.e_min + kPad) * trow;
     int EJ = g.tal[w], Mg = g.tal[2 * g.Wpad + w];
     // byte offsets of planes z - 1, z, z + 1 in shared memory
-    int am = ring ? 0 : (L - 1) * pb, az = ring ? pb : 0, ap = ring ? 2 * pb : pb;
+    int am = ring ? 0 : (L - 1) * pb, az = ring && !OWN ? pb : 0, ap = ring ? 2 * pb : pb;
+    // OWN: the lattice's bytes per row, the lanes' bytes of a row in it
+    const ptrdiff_t rsb = (ptrdiff_t)g.rw * g.wstr * 4;
+    const char *xg[SEG];
+#pragma unroll
+    for (int q = 0; q < SEG; ++q)
+        xg[q] = reinterpret_cast<const char *>(copy.g + (xo[q] >> 2) * g.wstr) + (xo[q] & 3);
 
     // random words of the four rows from site `site` on: block b of the walker
-    auto draw = [&](uint32_t *buf, int site, int n_blk, int b, uint64_t sw) {
-        const uint4 v = philox4x32_10(
+    auto draw = [&](int site, int b, uint64_t sw) {
+        return philox4x32_10(
             make_uint4((uint32_t)((site >> 2) + b), (uint32_t)sw, (uint32_t)(sw >> 32), 0u), keys);
-        st_shared_v4(shared_addr(buf + 4 * b), v, used && b < n_blk);
     };
+    auto keep = [&](uint32_t *to, uint4 v, int n_blk, int b) {
+        st_shared_v4(shared_addr(to + 4 * b), v, used && b < n_blk);
+    };
+    uint32_t *buf = mem, *buf1 = TWO ? mem + rows_random_words(L) : mem;
     auto blocks_of = [&](int site, int y0) {
         return ((site & 3) + min(4, L - y0) * L + 3) >> 2;
     };
-    uint32_t *buf = mem, *buf1 = mem + rows_random_words(L);
-    for (int b = h; b < blocks_of(0, 0); b += A) draw(buf, 0, blocks_of(0, 0), b, sweep0);
+    for (int b = h; b < blocks_of(0, 0); b += A) keep(mem, draw(0, b, sweep0), blocks_of(0, 0), b);
     cp_wait_all();
     __syncwarp();
 
@@ -259,6 +303,8 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
         for (int z = 0; z < L; ++z) {
             const uint2 *jrow = reinterpret_cast<const uint2 *>(g.J6) + z * L * L;
             const int dm = am - az, dp = ap - az;
+            const ptrdiff_t zm_o = (ptrdiff_t)(z ? z - 1 : L - 1) * L * rsb;
+            const ptrdiff_t zp_o = (ptrdiff_t)(z + 1 < L ? z + 1 : 0) * L * rsb;
             // per segment: the old spin of the next row to form, the new spin of
             // the row before the current one
             int own[SEG], ym[SEG];
@@ -278,6 +324,7 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                 int8_t *const row = sp + az + y0 * PITCH;
                 const uint32_t row_a = sp_a + az + y0 * PITCH;
                 const uint32_t *const rnd = buf + (site0 & 3);
+                uint4 drawn[SEG];
                 // The Site of row j, segment q, in two parts: the loads, and the
                 // rest.  x neighbours are the old spins (a step adds what the
                 // row changed), but for site L - 1 of a row of several segments,
@@ -289,12 +336,23 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                 };
                 auto load = [&](int j, int q) {
                     Raw r;
+                    // rows past the plane's last are formed (where there is no slack,
+                    // from its first row) and not used
+                    const int8_t *const rj = SEG == 1 || y0 + j < L ? row + j * PITCH : sp + az;
+                    const int8_t *const ru = SEG == 1 || y0 + j + 1 < L ? row + (j + 1) * PITCH
+                                             : sp + az + (REPEAT0 ? L * PITCH : 0);
                     r.rw = rnd[j * L + xo[q]];
-                    r.zm = (row + dm + j * PITCH)[xo[q]];
-                    r.zp = (row + dp + j * PITCH)[xo[q]];
-                    r.xl = (row + j * PITCH)[xl_o[q]];
-                    r.xr = (row + j * PITCH)[xr_o[q]];
-                    r.up = (row + (j + 1) * PITCH)[xo[q]];
+                    if (OWN) {
+                        const ptrdiff_t at = (ptrdiff_t)min(y0 + j, L - 1) * rsb;
+                        r.zm = ld_lattice(xg[q] + zm_o + at);
+                        r.zp = ld_lattice(xg[q] + zp_o + at);
+                    } else {
+                        r.zm = (rj + dm)[xo[q]];
+                        r.zp = (rj + dp)[xo[q]];
+                    }
+                    r.xl = rj[xl_o[q]];
+                    r.xr = rj[xr_o[q]];
+                    r.up = ru[xo[q]];
                     r.j = make_uint2(0u, 0u);
                     if (BONDS) r.j = __ldg(jrow + (y0 + j < L ? (y0 + j) * L : 0) + xo[q]);
                     return r;
@@ -328,11 +386,21 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                     }
                     return t;
                 };
+                // what a Site takes from the other lanes: issued beside the ballot
+                // of the step before, since every warp-wide operation ends a
+                // stretch of code that the compiler can interleave
+                auto gather = [&](Site &t) {
+                    t.dl = __shfl_sync(~0u, t.delta, (lane - 1) & 31);
+                    t.d0 = SEG == 1 ? __shfl_sync(~0u, t.delta, sbase) : 0;
+                    t.Pm = __ballot_sync(~0u, t.d > 0);
+                    t.Mm = __ballot_sync(~0u, t.d < 0);
+                };
                 // couplings to the y - 1, x - 1 and x + 1 neighbours
                 auto j_ym = [](const Site &t) { return BONDS ? (int)t.j >> 24 : 1; };
                 auto j_xl = [](const Site &t) { return BONDS ? (int)(int8_t)(t.j >> 8) : 1; };
                 auto j_xr = [](const Site &t) { return BONDS ? (int)(int8_t)t.j : 1; };
                 Site c = form(load(0, 0), 0);
+                gather(c);
                 int edge = 0;  // the change of the last site of the segment before
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -347,58 +415,74 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                         if (SEG > 1 && q > 0) hh += (h == 0 ? edge : 0) * j_xl(c);
                         const int hk0 = c.step * hh, row0 = eo + c.d * nj;
                         const uint32_t t0 = __ldg(thr + (row0 + hk0));
-                        // meanwhile: what the row's further passes need, the next
-                        // step's Site, the next four rows' random words
-                        const int dl = __shfl_sync(~0u, c.delta, (lane - 1) & 31);
-                        const int d0 = SEG == 1 ? __shfl_sync(~0u, c.delta, sbase) : 0;
-                        const unsigned Pm = __ballot_sync(~0u, c.d > 0);
-                        const unsigned Mm = __ballot_sync(~0u, c.d < 0);
-                        // changes of hk0 when the left neighbour (for site L - 1 also
-                        // site 0) is accepted
-                        const int cL = c.step * dl * j_xl(c), cW = c.step * d0 * j_xr(c);
-                        if (j == 0) draw(buf1, site_n, blk_n, q * A + h, sw_n);
+                        // meanwhile the next step's Site and the next four rows'
+                        // random words
+                        if (j == 0) {
+                            drawn[q] = draw(site_n, q * A + h, sw_n);
+                            if (TWO) keep(buf1, drawn[q], blk_n, q * A + h);
+                        }
                         Site n = c;
-                        if (jn < 4 && SEG == 1) n = form(r, qn);
+                        if (jn < 4) n = form(r, qn);
                         bool mine = c.u < t0;
                         unsigned acc = __ballot_sync(~0u, mine);
+                        const bool some = __any_sync(~0u, mine);
+                        if (jn < 4) gather(n);
                         edge = 0;
                         int s_new = c.s;
-                        if (__any_sync(~0u, mine)) {
-                            int hk, nd;
-                            bool again;
+                        if (some) {
+                            // hk0 changes by cL when the left neighbour is accepted, for
+                            // site L - 1 by cW when site 0 is, which the first pass
+                            // decided for good
+                            const int cL = c.step * c.dl * j_xl(c);
+                            int hb = hk0, hk;
+                            if (SEG == 1) hb += (acc & bit0) ? c.step * c.d0 * j_xr(c) : 0;
+                            bool was;
                             do {
-                                hk = hk0 + ((acc & bitL) ? cL : 0);
-                                if (SEG == 1) hk += (acc & bit0) ? cW : 0;
+                                was = mine;
+                                hk = hb + ((acc & bitL) ? cL : 0);
                                 // E_Delta moves by the accepted d before the site
-                                nd = __popc(acc & Pm & lower) - __popc(acc & Mm & lower);
+                                const int nd = __popc(acc & c.Pm & lower) - __popc(acc & c.Mm & lower);
                                 mine = c.u < __ldg(thr + (row0 + hk + nd * trow));
-                                const unsigned na = __ballot_sync(~0u, mine);
-                                again = na != acc;
-                                acc = na;
-                            } while (__any_sync(~0u, again));
+                                acc = __ballot_sync(~0u, mine);
+                            } while (__any_sync(~0u, mine != was));
                             // E_J changes by |delta| k h (clean), -delta h (couplings)
                             const int da = mine ? c.delta : 0;
                             dJ += BONDS ? (mine ? hk : 0) : hk * abs(da);
                             dM += da;
                             s_new += da;
                             st_shared_u8(row_a + j * PITCH + xo[q], s_new, mine);
-                            if (j == 0) st_shared_u8(row_a + L * PITCH + xo[q], s_new, mine && y0 == 0);
-                            nd += mine ? c.d : 0;
-                            const int end = q + 1 < SEG ? sbase + A - 1 : last_lane;
-                            eo += trow * __shfl_sync(~0u, nd, end);
-                            if (SEG > 1 && q + 1 < SEG) edge = __shfl_sync(~0u, da, end);
+                            if (j == 0 && REPEAT0 && !OWN)
+                                st_shared_u8(row_a + L * PITCH + xo[q], s_new, mine && y0 == 0);
+                            eo += trow * (__popc(acc & c.Pm & lanes) - __popc(acc & c.Mm & lanes));
+                            if (SEG > 1 && q + 1 < SEG) edge = __shfl_sync(~0u, da, sbase + A - 1);
                         }
+                        // (plane z's row 0 gives way to plane z + 1's: its copy is made here)
+                        if (j == 0 && OWN)
+                            st_shared_u8(row_a + L * PITCH + xo[q], s_new, y0 == 0 && !idle[q]);
                         ym[q] = s_new;
-                        if (jn < 4 && SEG > 1) n = form(r, qn);
                         c = n;
                     }
                 }
-                if (blk_n > SEG * A) draw(buf1, site_n, blk_n, SEG * A + h, sw_n);
+                if (!TWO) {
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < SEG; ++q) keep(buf1, drawn[q], blk_n, q * A + h);
+                }
+                if (blk_n > SEG * A)
+                    keep(buf1, draw(site_n, SEG * A + h, sw_n), blk_n, SEG * A + h);
                 __syncwarp();
                 // the finished rows back to the lattice, and the same rows of plane
                 // z + 2 over those of plane z - 1
+                if (OWN && wide) {
+                    // the z + 1 rows, first touched by the steps above, eight rows
+                    // ahead from HBM into L2 (64 bytes per lane)
+                    const ptrdiff_t at = zp_o + (ptrdiff_t)(y0 + 8) * PITCH + 64 * h;
+                    prefetch_l2(reinterpret_cast<const char *>(copy.g) + at,
+                                used && 64 * h < 4 * PITCH && at < (ptrdiff_t)L * L * PITCH);
+                }
                 if (ring) {
-                    const int n = min(4, L - y0), z2 = z + 2 < L ? z + 2 : z + 2 - L;
+                    const int n = min(4, L - y0), zn = z + (OWN ? 1 : 2), z2 = zn < L ? zn : zn - L;
+                    const int dv = OWN ? 0 : dm;  // the rows that give way
                     if (wide) {
                         // n PITCH bytes, 16 per lane and turn
                         const ptrdiff_t o = (ptrdiff_t)(z * L + y0) * PITCH;
@@ -410,25 +494,32 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                             const uint4 v =
                                 *reinterpret_cast<const uint4 *>(row + (p ? 16 * h + at : 0));
                             st_global_v4(lat + o + at, v, p);
-                            cp16(row_a + dm + 16 * h + at, lat + i + at, p);
-                            if (t == 0)
-                                cp16(row_a + dm + L * PITCH + 16 * h, lat + i,
+                            cp16(row_a + dv + 16 * h + at, lat + i + at, p);
+                            if (t == 0 && REPEAT0 && !OWN)
+                                cp16(row_a + dv + L * PITCH + 16 * h, lat + i,
                                      used && y0 == 0 && 16 * h < PITCH);
                         }
                     } else if (used) {
                         copy.out(row, z, y0, n);
-                        copy.in(row + dm, z2, y0, n);
-                        if (y0 == 0) copy.in(row + dm + L * PITCH, z2, 0, 1);
+                        copy.in(row + dv, z2, y0, n);
+                        if (REPEAT0 && !OWN && y0 == 0) copy.in(row + dv + L * PITCH, z2, 0, 1);
                     }
                     cp_commit();
                     cp_wait_1();
                     __syncwarp();
                 }
-                uint32_t *const t = buf;
-                buf = buf1;
-                buf1 = t;
+                if (TWO) {
+                    uint32_t *const t = buf;
+                    buf = buf1;
+                    buf1 = t;
+                }
             }
             // the next plane
+            if (OWN) {
+                cp_wait_all();  // its last rows came in just now
+                __syncwarp();
+                continue;
+            }
             const int t = am;
             am = az;
             az = ap;
@@ -503,7 +594,7 @@ int rows_lattice_words(int L) { return rows_slots(L) < L ? rows_pitch(L) / 4 : (
 size_t rows_bytes_for(int L)
 {
     const RowShape s = rows_shape(L);
-    return (size_t)s.per_warp * rows_walker_words(L, s.per_warp, rows_pitch(L)) * sizeof(uint32_t);
+    return (size_t)s.per_warp * rows_walker_words(L, s.seg, s.per_warp, rows_pitch(L)) * sizeof(uint32_t);
 }
 
 namespace {
