@@ -41,14 +41,14 @@
 // Measured on GB300 against the kernels that the autotuner picked before
 // (sweep.cu's split kernel for L = 8 .. 32, scan.cu's for L = 48, one thread
 // per walker for L % 4 != 0 and for couplings), time per call:
-//   L = 8, T = 2, 64 walkers, 200 sweeps and merge    11.7 -> 4.4 ms
-//   L = 16, T = 1, 1024 walkers, 500 sweeps and merge 94.3 -> 24.6 ms
-//   L = 32, T = 0.9, 2048 walkers, 150 and merge      156 -> 43.9 ms
+//   L = 8, T = 2, 64 walkers, 200 sweeps and merge    11.8 -> 4.4 ms
+//   L = 16, T = 1, 1024 walkers, 500 sweeps and merge 94.8 -> 24.6 ms
+//   L = 32, T = 0.9, 2048 walkers, 150 and merge      157 -> 43.4 ms
 //   L = 8 .. 32 in one context, 12288 walkers, 60     112 -> 43.5 ms
 //   L = 22, T = 1.4182, 1000 walkers, 50 and merge    76.9 -> 6.8 ms
 //   L = 28, T = 1, 1024 walkers, 100 recorded         74.4 -> 26.0 ms
-//   L = 48, T = 0.9, 4096 walkers, 60 recorded        254 -> 157 ms
-//   couplings, L = 24, 4096 walkers, 50 and merge     120 -> 24.7 ms
+//   L = 48, T = 0.9, 4096 walkers, 60 recorded        248 -> 115 ms
+//   couplings, L = 24, 4096 walkers, 50 and merge     120 -> 23.4 ms
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -128,15 +128,14 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 __device__ __forceinline__ void cp_wait_1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// How a walker's rows pass through shared memory, by the number of segments
-// (L <= 32: 1, L <= 48: 3, above: 4).
-//   planes: up to 12 sites all L; one and three segments the three planes that
+// How a walker's rows pass through shared memory, by the number of segments.
+//   planes: up to 12 sites all L; one to three segments the three planes that
 //     a row reads (z - 1, z, z + 1); four segments plane z alone, whose finished
 //     rows give way to those of plane z + 1, the z neighbours read from the
 //     lattice a step ahead;
 //   row L of a plane repeats row 0, the y + 1 neighbour of the last row, but for
 //     three segments, where a select takes its place;
-//   random words: two buffers for one segment, so that the next rows' words are
+//   random words: two buffers for one or two segments, so that the next rows' words are
 //     stored as they are drawn; else one, the words waiting in registers.
 // The differences buy room: 48-site rows take 15.5 KB per warp, 14 warps per
 // SM, so that the benchmark's 2048 warps run in one wave (17.4 KB left 72 of
@@ -144,19 +143,19 @@ __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;
 // plane z alone, the z neighbours' latency gave 146 ms).
 // Rows are PITCH bytes apart, so a row's addresses are a register and a
 // constant.
-__host__ __device__ constexpr int rows_slots(int L) { return L <= 12 ? L : L <= 48 ? 3 : 1; }
+__host__ __device__ constexpr int rows_slots(int L, int seg) { return L <= 12 ? L : seg <= 3 ? 3 : 1; }
 __host__ __device__ constexpr bool rows_repeat0(int seg) { return seg != 3; }
-__host__ __device__ constexpr int rows_buffers(int seg) { return seg == 1 ? 2 : 1; }
+__host__ __device__ constexpr int rows_buffers(int seg) { return seg <= 2 ? 2 : 1; }
 // Words of a buffer: four rows touch at most L + 1 Philox blocks (rows that
 // start inside a block, L odd, one more than L).
 __host__ __device__ constexpr int rows_random_words(int L) { return 4 * (L + 1); }
 // Words from one walker to the next: 16-byte aligned, and spread over the
 // banks so that the walkers of a warp read a row without conflicts.  With one
-// segment the rows after a plane's last are read, and not used: two rows of
+// or two segments the rows after a plane's last are read, and not used: two rows of
 // slack.
 __host__ __device__ inline int rows_walker_words(int L, int seg, int per_warp, int pitch)
 {
-    const int rows = rows_slots(L) * (L + rows_repeat0(seg)) + (seg == 1 ? 2 : 0);
+    const int rows = rows_slots(L, seg) * (L + rows_repeat0(seg)) + (seg <= 2 ? 2 : 0);
     const int n = rows_buffers(seg) * rows_random_words(L) + rows * (pitch / 4);
     const int want = per_warp <= 1 ? 0 : per_warp == 2 ? 16 : per_warp <= 4 ? 8 : 4;
     return want ? n + ((want - n) % 32 + 32) % 32 : (n + 3) / 4 * 4;
@@ -237,7 +236,7 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
     int8_t *const sp = reinterpret_cast<int8_t *>(mem + rows_buffers(SEG) * rows_random_words(L));
     constexpr bool REPEAT0 = rows_repeat0(SEG), TWO = rows_buffers(SEG) == 2;
     const int pb = (L + REPEAT0) * PITCH;  // bytes per plane
-    const bool ring = rows_slots(L) < L;
+    const bool ring = rows_slots(L, SEG) < L;
     constexpr bool OWN = SEG > 3;  // plane z alone in shared memory
     const RowCopy<PITCH> copy{g.spins + (ptrdiff_t)w * g.cstr, g.wstr, L, g.Lw, g.rw, h};
     // a lattice whose rows lie as in shared memory is copied 16 bytes per lane
@@ -327,8 +326,8 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                 uint4 drawn[SEG];
                 // The Site of row j, segment q, in two parts: the loads, and the
                 // rest.  x neighbours are the old spins (a step adds what the
-                // row changed), but for site L - 1 of a row of several segments,
-                // whose right neighbour, site 0, is final by then.
+                // row changed), but for site L - 1 of a row of three or more
+                // segments, whose right neighbour, site 0, is final by then.
                 struct Raw {
                     uint32_t rw;
                     int zm, zp, xl, xr, up;
@@ -338,8 +337,8 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                     Raw r;
                     // rows past the plane's last are formed (where there is no slack,
                     // from its first row) and not used
-                    const int8_t *const rj = SEG == 1 || y0 + j < L ? row + j * PITCH : sp + az;
-                    const int8_t *const ru = SEG == 1 || y0 + j + 1 < L ? row + (j + 1) * PITCH
+                    const int8_t *const rj = SEG <= 2 || y0 + j < L ? row + j * PITCH : sp + az;
+                    const int8_t *const ru = SEG <= 2 || y0 + j + 1 < L ? row + (j + 1) * PITCH
                                              : sp + az + (REPEAT0 ? L * PITCH : 0);
                     r.rw = rnd[j * L + xo[q]];
                     if (OWN) {
@@ -362,7 +361,7 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                     t.s = own[q];
                     own[q] = r.up;
                     int xr = r.xr;
-                    if (SEG > 1 && q == SEG - 1) {
+                    if (SEG > 2 && q == SEG - 1) {
                         const int er = __shfl_sync(~0u, ym[0], sbase);
                         xr = lane == last_lane ? er : xr;
                     }
@@ -401,7 +400,8 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                 auto j_xr = [](const Site &t) { return BONDS ? (int)(int8_t)t.j : 1; };
                 Site c = form(load(0, 0), 0);
                 gather(c);
-                int edge = 0;  // the change of the last site of the segment before
+                // changes of the last site of the segment before, of site 0
+                int edge = 0, first = 0;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     if (j > 0 && y0 + j >= L) break;
@@ -413,6 +413,7 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                         // first pass: nothing accepted before the site
                         int hh = c.h + ym[q] * j_ym(c);
                         if (SEG > 1 && q > 0) hh += (h == 0 ? edge : 0) * j_xl(c);
+                        if (SEG == 2 && q == 1) hh += (lane == last_lane ? first : 0) * j_xr(c);
                         const int hk0 = c.step * hh, row0 = eo + c.d * nj;
                         const uint32_t t0 = __ldg(thr + (row0 + hk0));
                         // meanwhile the next step's Site and the next four rows'
@@ -428,6 +429,7 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                         const bool some = __any_sync(~0u, mine);
                         if (jn < 4) gather(n);
                         edge = 0;
+                        if (q == 0) first = 0;
                         int s_new = c.s;
                         if (some) {
                             // hk0 changes by cL when the left neighbour is accepted, for
@@ -455,6 +457,7 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                                 st_shared_u8(row_a + L * PITCH + xo[q], s_new, mine && y0 == 0);
                             eo += trow * (__popc(acc & c.Pm & lanes) - __popc(acc & c.Mm & lanes));
                             if (SEG > 1 && q + 1 < SEG) edge = __shfl_sync(~0u, da, sbase + A - 1);
+                            if (SEG == 2 && q == 0) first = __shfl_sync(~0u, da, sbase);
                         }
                         // (plane z's row 0 gives way to plane z + 1's: its copy is made here)
                         if (j == 0 && OWN)
@@ -488,7 +491,7 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                         const ptrdiff_t o = (ptrdiff_t)(z * L + y0) * PITCH;
                         const ptrdiff_t i = (ptrdiff_t)(z2 * L + y0) * PITCH;
 #pragma unroll
-                        for (int t = 0; t < (SEG == 1 ? 1 : 2); ++t) {
+                        for (int t = 0; t < (SEG <= 2 ? 1 : 2); ++t) {
                             const int at = t * 16 * A;
                             const bool p = used && 16 * h + at < n * PITCH;
                             const uint4 v =
@@ -574,12 +577,17 @@ sweep_rows_kernel(const __grid_constant__ GroupDev g, int lanes, uint32_t seed, 
 
 }  // namespace
 
-// Segments and lanes of a row of L sites.
-RowShape rows_shape(int L)
+// Segments and lanes of a row of L sites, for a group of W walkers.  Rows of up
+// to 32 sites are one segment.  Longer rows fill their warps best with three
+// segments of up to 16 lanes (L <= 48) or four, two walkers per warp; while the
+// walkers are fewer than the 608 schedulers, lanes are to spare and the time is
+// that of a row, so two segments and one walker per warp (L = 48: 608 walkers
+// on two segments 0.77 ms a sweep, 640 on three 1.34 ms).
+RowShape rows_shape(int L, int W)
 {
     RowShape s{0, 0, 0};
     if (L < 3 || L > 64) return s;
-    s.seg = L <= 32 ? 1 : L <= 48 ? 3 : 4;
+    s.seg = L <= 32 ? 1 : W <= 608 ? 2 : L <= 48 ? 3 : 4;
     s.lanes = (L + s.seg - 1) / s.seg;
     s.per_warp = 32 / s.lanes;
     return s;
@@ -589,12 +597,12 @@ RowShape rows_shape(int L)
 // kept walker by walker whose planes pass through it (rows_lattice_words).
 static int rows_pitch(int L) { return L <= 16 ? 16 : L <= 32 ? 32 : L <= 48 ? 48 : 64; }
 
-int rows_lattice_words(int L) { return rows_slots(L) < L ? rows_pitch(L) / 4 : (L + 3) / 4; }
+int rows_lattice_words(int L) { return L > 12 ? rows_pitch(L) / 4 : (L + 3) / 4; }
 
-size_t rows_bytes_for(int L)
+static size_t rows_bytes_for(int L, const RowShape &s)
 {
-    const RowShape s = rows_shape(L);
-    return (size_t)s.per_warp * rows_walker_words(L, s.seg, s.per_warp, rows_pitch(L)) * sizeof(uint32_t);
+    return (size_t)s.per_warp * rows_walker_words(L, s.seg, s.per_warp, rows_pitch(L)) *
+           sizeof(uint32_t);
 }
 
 namespace {
@@ -615,15 +623,23 @@ cudaError_t launch_sweeps_rows(const GroupDev &g, uint32_t seed, uint64_t sweep0
                                int64_t ts_pos, bool record, cudaStream_t st)
 {
     if (n_sweeps <= 0) return cudaSuccess;
-    const RowShape sh = rows_shape(g.L);
+    const RowShape sh = rows_shape(g.L, g.W);
     if (sh.seg == 0) return cudaErrorInvalidValue;
     const int blocks = (g.W + sh.per_warp - 1) / sh.per_warp, rec = record ? 1 : 0;
-    const size_t smem = rows_bytes_for(g.L);  // at most 28 KB: no opt-in
-    switch (rows_pitch(g.L)) {
-        case 16: launch<1, 16>(g, sh, blocks, smem, seed, sweep0, n_sweeps, ts_pos, rec, st); break;
-        case 32: launch<1, 32>(g, sh, blocks, smem, seed, sweep0, n_sweeps, ts_pos, rec, st); break;
-        case 48: launch<3, 48>(g, sh, blocks, smem, seed, sweep0, n_sweeps, ts_pos, rec, st); break;
-        default: launch<4, 64>(g, sh, blocks, smem, seed, sweep0, n_sweeps, ts_pos, rec, st); break;
+    const size_t smem = rows_bytes_for(g.L, sh);  // at most 16 KB: no opt-in
+    switch (sh.seg * 100 + rows_pitch(g.L)) {
+#define MUCA_ROWS_LAUNCH(S, P)                                                          \
+    case S * 100 + P:                                                                   \
+        launch<S, P>(g, sh, blocks, smem, seed, sweep0, n_sweeps, ts_pos, rec, st);     \
+        break;
+        MUCA_ROWS_LAUNCH(1, 16)
+        MUCA_ROWS_LAUNCH(1, 32)
+        MUCA_ROWS_LAUNCH(2, 48)
+        MUCA_ROWS_LAUNCH(2, 64)
+        MUCA_ROWS_LAUNCH(3, 48)
+        MUCA_ROWS_LAUNCH(4, 64)
+#undef MUCA_ROWS_LAUNCH
+        default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }

@@ -414,7 +414,7 @@ int upload_groups(muca_ctx *ctx)
 // Whether the site-per-lane kernel sweeps the group.
 bool on_rows(const Group &g)
 {
-    return rows_shape(g.L).seg > 0 && (g.jmax > 0 || g.residency == MUCA_RES_ROWS);
+    return rows_shape(g.L, g.W).seg > 0 && (g.jmax > 0 || g.residency == MUCA_RES_ROWS);
 }
 
 // Kernel kind of a group's block list (-1: none, the site-per-lane kernel).
@@ -691,8 +691,8 @@ static int tune_group(muca_ctx *ctx, size_t gi, int residency, int wpb, int P)
     Group &g = ctx->g[gi];
     if (g.by_walker) {
         g.residency = MUCA_RES_ROWS;
-        g.wpb = rows_shape(g.L).per_warp;
-        g.P = rows_shape(g.L).lanes;
+        g.wpb = rows_shape(g.L, g.W).per_warp;
+        g.P = rows_shape(g.L, g.W).lanes;
         return MUCA_OK;
     }
     const int smem_max = max_smem_per_block();
@@ -1044,7 +1044,7 @@ int muca_init(const muca_group *groups, int n_groups, const muca_options *opt, v
             g.beta = 1.0 / g.T;
             g.walker0 = w0 + (uint32_t)lo;
             g.by_walker = opt->residency == MUCA_RES_AUTO && opt->walkers_per_block == 0 &&
-                          opt->lanes_per_walker == 0 && rows_shape(g.L).seg > 0;
+                          opt->lanes_per_walker == 0 && rows_shape(g.L, g.W).seg > 0;
             w0 += (uint32_t)tot;
             g.lnW.assign(g.nE, 0.0);
             g.acc.assign((size_t)std::max(g.nE - 1, 1), 0.0);
@@ -1644,13 +1644,14 @@ int muca_get_state(muca_ctx *ctx, int group, int8_t *spins, int32_t *tallies)
         CK(cudaMemcpyAsync(dev.data(), g.spins, dev.size() * sizeof(uint32_t),
                            cudaMemcpyDeviceToHost, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
+        const size_t step = g.by_walker ? 1 : g.Wpad;
         for (int w = 0; w < g.W; ++w)
-            for (int row = 0; row < g.L * g.L; ++row)
-                for (int x = 0; x < g.L; ++x) {
-                    const uint32_t word = dev[word_at(g, row, x >> 2, w)];
-                    spins[(size_t)w * g.V + (size_t)row * g.L + x] =
-                        (int8_t)(uint8_t)(word >> (8 * (x & 3)));
-                }
+            for (int row = 0; row < g.L * g.L; ++row) {
+                const uint32_t *src = dev.data() + word_at(g, row, 0, w);
+                int8_t *dst = spins + (size_t)w * g.V + (size_t)row * g.L;
+                for (int x = 0; x < g.L; ++x)
+                    dst[x] = (int8_t)(uint8_t)(src[(x >> 2) * step] >> (8 * (x & 3)));
+            }
     }
     if (tallies) {
         std::vector<int32_t> t((size_t)3 * g.Wpad);
@@ -1670,16 +1671,19 @@ int muca_set_state(muca_ctx *ctx, int group, const int8_t *spins)
     if (!spins) return fail(ctx, MUCA_ERR_INVALID_ARG, "spins is NULL");
     Group &g = ctx->g[group];
     std::vector<uint32_t> dev(lattice_words(g), 0u);
+    const size_t step = g.by_walker ? 1 : g.Wpad;
     for (int w = 0; w < g.W; ++w)
-        for (int row = 0; row < g.L * g.L; ++row)
+        for (int row = 0; row < g.L * g.L; ++row) {
+            const int8_t *src = spins + (size_t)w * g.V + (size_t)row * g.L;
+            uint32_t *dst = dev.data() + word_at(g, row, 0, w);
             for (int x = 0; x < g.L; ++x) {
-                const int8_t s = spins[(size_t)w * g.V + (size_t)row * g.L + x];
+                const int8_t s = src[x];
                 if (s < -1 || s > 1)
                     return fail(ctx, MUCA_ERR_INVALID_ARG, "walker %d site %d: spin %d", w,
                                 row * g.L + x, s);
-                dev[word_at(g, row, x >> 2, w)] |=
-                    (uint32_t)(uint8_t)s << (8 * (x & 3));
+                dst[(x >> 2) * step] |= (uint32_t)(uint8_t)s << (8 * (x & 3));
             }
+        }
     std::vector<int32_t> old((size_t)3 * g.Wpad);
     std::vector<uint32_t> old_spins(dev.size());
     CK(cudaMemcpyAsync(old.data(), g.tal, old.size() * sizeof(int32_t), cudaMemcpyDeviceToHost,
@@ -1722,7 +1726,7 @@ int muca_get_config(muca_ctx *ctx, int group, int32_t *residency, int32_t *walke
     int rc = check_group_index(ctx, group);
     if (rc) return rc;
     const Group &g = ctx->g[group];
-    const RowShape rows = rows_shape(g.L);
+    const RowShape rows = rows_shape(g.L, g.W);
     const bool lane = g.jmax && on_rows(g);  // couplings on the site-per-lane kernel
     if (residency) *residency = g.jmax ? MUCA_RES_BONDS : g.residency;
     if (walkers_per_block)

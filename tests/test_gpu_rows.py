@@ -1,7 +1,7 @@
 """The site-per-lane sweep kernel (the choice of MUCA_RES_AUTO) against the
 oracle, bit for bit: every way a row is laid out on a warp (one segment, rows
-that are no multiple of 4, the last length of each shared-memory row width,
-three and four segments with full and ragged last ones), the hot regime in
+that are no multiple of 4, the last length of each shared-memory row width, two
+to four segments with full and ragged last ones), the hot regime in
 which a row takes many passes, narrow windows, and checkpoints between its
 lattice layout and the walker-minor one."""
 import numpy as np
@@ -21,7 +21,8 @@ def muca():
     return m
 
 
-def run_against_oracle(L, T, W, lnW, n, bonds=None, e_min=0, e_max=None, spins0=None):
+def run_against_oracle(L, T, W, lnW, n, bonds=None, e_min=0, e_max=None, spins0=None,
+                       walkers=None):
     V = L ** 3
     e_max = V if e_max is None else e_max
     c = muca().Context([{"L": L, "T": T, "n_walkers": W, "e_min": e_min, "e_max": e_max}], seed=L)
@@ -40,7 +41,7 @@ def run_against_oracle(L, T, W, lnW, n, bonds=None, e_min=0, e_max=None, spins0=
     jmax = None if bonds is None else int(np.abs(bonds).max())
     thr = (oracle.build_table(L, T, e_min, e_max, lnW) if bonds is None else
            oracle.build_table_bonds(L, T, jmax, e_min, e_max, lnW))
-    for w in range(W):
+    for w in walkers or range(W):
         sp = oracle.init_spins(L, L, w) if spins0 is None else spins0[w].copy()
         if bonds is None:
             t = oracle.energies(L, sp).astype(np.int32)
@@ -65,6 +66,17 @@ def test_every_row_layout_under_rough_transition_weights(L, W):
     T = 1.0
     lnW = -2.944 / T * np.arange(L ** 3 + 1) + wl.random_lnW(L ** 3 + 1, L, scale=0.5)
     run_against_oracle(L, T, W, lnW, 3 if L <= 33 else 2)
+
+
+@pytest.mark.parametrize("L,jj", [(33, None), (48, None), (49, None), (64, None), (40, (1, 3)),
+                                  (52, (-1, 2))])
+def test_long_rows_of_many_walkers(L, jj):
+    """More than 608 walkers: rows beyond 32 sites in three or four segments, two
+    walkers per warp (fewer walkers take two segments); sampled walkers."""
+    V = L ** 3
+    lnW = -1.5 * np.arange(V + 1) + wl.random_lnW(V + 1, L, scale=0.5)
+    run_against_oracle(L, 3.0, 611, lnW, 2, walkers=[0, 1, 2, 305, 609, 610],
+                       bonds=None if jj is None else wl.random_bonds(L, jj[0], jj[1], seed=L))
 
 
 @pytest.mark.parametrize("L,W,jj", [(3, 12, (1, 3)), (7, 6, (-1, 1)), (12, 5, (2, 8)),
