@@ -409,7 +409,7 @@ def run_ours(args, rank, world, local_rank):
             "config": {"workload": "L=48 T=0.9 4096 walkers: 1000-sweep MUCA iteration "
                                    "(graph) + 250 recorded sweeps + FP32 reweight to 4096 Delta",
                        "L": L, "T": T, "walkers": W, "sweeps_per_step": sweeps + meas,
-                       "residency": {1: "global", 2: "smem", 3: "split", 4: "scan"}.get(res, str(res)),
+                       "residency": {1: "global", 2: "smem", 3: "split", 4: "scan", 6: "rows"}.get(res, str(res)),
                        "walkers_per_block": wpb, "lanes_per_walker": lanes, "seed": s["seed"],
                        "l2": "inputs larger than L2 (lattice 453 MB int8)"},
             "plain": {"value": plain_value, "unit": UNIT, "steps": plain_steps},
@@ -418,7 +418,8 @@ def run_ours(args, rank, world, local_rank):
                          "traffic": traffic_per_launch(res, sweeps),
                          "kernel": {1: "sweep_global_kernel<false>", 2: "sweep_smem_kernel<false>",
                                     3: "sweep_ws_kernel<false, true>",
-                                    4: f"sweep_scan_kernel<{L}>"}.get(res, str(res)),
+                                    4: f"sweep_scan_kernel<{L}>",
+                                    6: "sweep_rows_kernel<3, 48, false>"}.get(res, str(res)),
                          "ops_per_attempt": ops_per_attempt,
                          "peak_source": f"measured: muca_probe_int, {int_kind}, "
                                         f"{probes['sm_count']} SMs x 8 blocks x 256 threads "
@@ -512,7 +513,7 @@ def mixed_bench(torch, muca, stream, n_it=2, n_full=None):
             "unit": UNIT, "batched": vfull, "batched_ms": ms_b + ms_rest,
             f"batched_first_{n_it}": vb, "plain_per_config_first": vp,
             "batched_over_plain_first": vb / vp, "plain_ms_first": ms_p,
-            "batched_configs": [{"residency": {1: "global", 2: "smem", 3: "split", 4: "scan"}.get(c[0], str(c[0])),
+            "batched_configs": [{"residency": {1: "global", 2: "smem", 3: "split", 4: "scan", 6: "rows"}.get(c[0], str(c[0])),
                                  "walkers_per_block": c[1], "lanes_per_walker": c[2]}
                                 for c in cfgs]}
 
@@ -554,7 +555,7 @@ def disordered_bench(torch, muca, stream):
     return {"workload": f"L={d['L']} T={d['T']} {d['n_walkers']} walkers, bimodal couplings "
                         f"{d['j1']}/{d['j2']} (p = 1/2), one iteration of {d['sweeps']} sweeps",
             "unit": UNIT, "value": attempts / (ms_graph / 1e3), "kernel_ms": k_ms,
-            "kernel": "sweep_bonds_kernel", "residency": cfg[0],
+            "kernel": "sweep_rows_kernel<1, 32, true>", "residency": cfg[0],
             "roofline": {"bound": "hbm", "achieved_gbs": gbs, "peak_gbs": hbm,
                          "frac": gbs / hbm, "peak_kind": pk_kind, "bytes_per_attempt": 2}}
 
