@@ -6,14 +6,14 @@
 // works in two stages:
 //   A. one streaming pass over the samples accumulates, per E_Delta bin, exact
 //      integer sums: count, sum E_J, sum |M|, sum M^2 and sum M^4 (128-bit);
-//   B. for every Delta_k, a pass over the occupied bins: shift the exponents by
-//      their maximum, exponentiate, and form the weighted sums; C and chi are
-//      taken as centred second passes, so no difference of large moments is
-//      ever formed.
-// Stage B runs in FP64, or in FP32 where the exponent -beta Delta_k E - lnW(E)
-// is carried as a float pair (hi + lo, error-free products and sums) so that
-// its O(10^5) magnitude does not eat the 24-bit mantissa, and all sums are
-// Kahan-compensated.
+//   B. for every Delta_k, the weighted sums over the occupied bins, the exponents
+//      shifted by their maximum; C and chi are taken about the means, or about
+//      a bin that holds a good share of the weight, so no difference of large
+//      moments is ever formed.
+// Stage B runs in FP64 (blocks of bins), or in FP32 (bin by bin) where the
+// exponent -beta Delta_k E - lnW(E) is carried as a float pair (hi + lo,
+// error-free products and sums) so that its O(10^5) magnitude does not eat the
+// 24-bit mantissa, and all sums are Kahan-compensated.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -759,23 +759,30 @@ grid_kernel_f32(BinStats<float> s, int nE, int e_min, float beta, int V,
 
 // ------------------------------------------------------------ FP64 stage B
 // The weight of Eq. 3 factorises over a block of B consecutive bins: with
-// r = E - E_b the distance from the block's reference bin and s a slope common
-// to the grid,
-//   exp(-c E - lnW(E)) = A(c, b) exp(-(c - s) r) V(E),   c = beta Delta_k,
-//   A = exp(-c E_b - lnW(E_b) + v_b),  V = exp(-s r - (lnW(E) - lnW(E_b)) - v_b),
-// where v_b makes the block's largest V one.  V does not depend on the field,
-// and |c - s| B / 2 is small for a grid of fields around a transition.  So the
-// middle factor is its Taylor polynomial in x = -(c - s) B / 2, and each
-// weighted sum over the block is a polynomial in x whose coefficients sum
-// V f(E) (2 r / B)^p / p! over the block once per call: one exponential and
-// 8 deg multiply-adds per (field, block).  FP64 runs at two multiply-adds per
-// clock and SM here, so FP64 instructions are the time: bin by bin, with two
-// exponentials and eight compensated sums, they were about a hundred per
-// (field, bin); in blocks of 64 bins they are four.
-// The exponent of A is formed with error-free products and differences; sums
-// are taken about references near the bins (the block's means, then those of
-// the thread's first block), and the centred sums of C and chi follow from them
-// once the means are known, so no difference of large moments is formed.
+// E_b the block's heaviest bin (the largest n exp(-s E - lnW), s a slope common
+// to the grid) and r = E - E_b,
+//   exp(-c E - lnW(E)) = A(c, b) exp(-(c - s) (E - E_mid)) V(E),   c = beta Delta_k,
+//   A = exp(-c E_b - lnW(E_b) - (c - s) (E_mid - E_b)),
+//   V = exp(-s r - (lnW(E) - lnW(E_b))).
+// V does not depend on the field, and |c - s| B / 2 is small for a grid of
+// fields around a transition.  So the middle factor is its Taylor polynomial in
+// x = -(c - s) B / 2 (E_mid: the block's middle), and each weighted sum over
+// the block is a polynomial in x whose coefficients sum
+// V f(E) (2 (E - E_mid) / B)^p / p! over the block once per call: one
+// exponential and 8 deg multiply-adds per (field, block).  FP64 runs at two
+// multiply-adds per clock and SM here, so FP64 instructions are the time: bin
+// by bin, with two exponentials and eight compensated sums, they were about a
+// hundred per (field, bin); in blocks of 64 bins they are four.
+// The exponent of A is formed with error-free products and differences.  Sums
+// are taken about bins that hold weight, so that no difference of large moments
+// is formed, however narrow the distribution: inside a block about its heaviest
+// bin and its weighted mean E_J and |m|, across blocks about the heaviest
+// block's of the field.  (A reference that holds a share p of the weight lies
+// within 1 / sqrt(p) standard deviations of the mean.)
+//   C of a distribution pinned at one end of E_Delta (weights -ln of the binomial
+//   density of states, beta Delta = -25 .. 25) against binary128: within 7e-15,
+//   as with compensated sums about the mean; about the blocks' middle bins and
+//   the first blocks that count it was up to 1e-4
 //   4.1e7 samples, 32769 bins, 4096 fields: 21.8 -> 1.69 ms per call (bin by bin,
 //   then this), of which stage A 0.42, the coefficients 0.03, the fields 1.0 ms
 // FP32 keeps one evaluation per bin: its pipe is 64 times wider, and sums about
@@ -834,14 +841,14 @@ __host__ __device__ inline int block_slot(const BlockPlan &p, int b)
     return (b % p.per) * kRgThreads + b / p.per;
 }
 
-// Per slot: polynomial coefficients [deg + 1][kStats][slots]; the reference
-// bin's E_Delta and lnW, the block's mean E_J and |m|, its samples.
+// Per slot: polynomial coefficients [deg + 1][kStats][slots]; the block's
+// heaviest bin, its weighted mean E_J and |m|.
 struct Blocks {
     double *coef, *mj, *mm;
-    double *lw;  // lnW at the reference bin
-    double *v;   // v_b
+    double *lw;  // lnW at the heaviest bin
+    double *ln;  // ln of its samples, -inf for a block without samples
     int *E;      // its E_Delta
-    int *used;   // whether the block has samples
+    int *mid;    // E_mid - E_b
 };
 
 size_t block_bytes(const BlockPlan &p)
@@ -855,12 +862,12 @@ Blocks block_layout(const BlockPlan &p, char *mem)
     const size_t slots = (size_t)p.per * kRgThreads;
     Blocks b;
     b.lw = (double *)mem;
-    b.v = b.lw + slots;
-    b.coef = b.v + slots;
+    b.ln = b.lw + slots;
+    b.coef = b.ln + slots;
     b.mj = b.coef + slots * kStats * (p.deg + 1);
     b.mm = b.mj + slots;
     b.E = (int *)(b.mm + slots);
-    b.used = b.E + slots;
+    b.mid = b.E + slots;
     return b;
 }
 
@@ -869,62 +876,79 @@ __constant__ double inv_q[kDegMax + 1] = {
     0.0, 1.0, 1.0 / 2, 1.0 / 3, 1.0 / 4, 1.0 / 5, 1.0 / 6, 1.0 / 7, 1.0 / 8, 1.0 / 9, 1.0 / 10,
     1.0 / 11, 1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17, 1.0 / 18, 1.0 / 19, 1.0 / 20};
 
-// One block of bins per CTA: the statistics about the block's means, times V,
-// then thread (p, j) sums its coefficient.
+// One block of bins per CTA: its heaviest bin, the statistics about that bin
+// and the block's weighted means, times V, then thread (p, j) sums its
+// coefficient.
 __global__ void __launch_bounds__(192)
 block_coef_kernel(BinStats<double> s, int nE, int e_min, BlockPlan p, Blocks out)
 {
     __shared__ double f[kStats][64], t[kDegMax + 1][64];
-    __shared__ double sn[64], sj[64], sm[64], sv[64];
+    __shared__ double sv[64], sj[64], sm[64];
+    __shared__ int sa[64];
     const int b = blockIdx.x, e0 = b * p.B, len = min(p.B, nE - e0), i = threadIdx.x;
-    const int ref = min(e0 + p.B / 2, nE - 1), slot = block_slot(p, b);
-    const int r = e0 + i - ref;
-    const double lref = s.lw[ref];
-    double n = 0.0, mej = 0.0, cm = 0.0, a = -INFINITY;
+    const int mid = min(e0 + p.B / 2, nE - 1), slot = block_slot(p, b);
+    const double n = i < len ? s.n[e0 + i] : 0.0;
     if (i < 64) {
-        if (i < len) n = s.n[e0 + i];
-        if (n > 0.0) {
-            mej = s.mej[e0 + i];
-            cm = s.cm[e0 + i];
-            a = -(p.slope * (double)r) - (s.lw[e0 + i] - lref);
+        sv[i] = n > 0.0 ? (-(p.slope * (double)(e0 + i - mid)) - (s.lw[e0 + i] - s.lw[mid])) + log(n)
+                        : -INFINITY;
+        sa[i] = i;
+    }
+    __syncthreads();
+    for (int o = 32; o > 0; o >>= 1) {
+        if (i < o && sv[i + o] > sv[i]) {
+            sv[i] = sv[i + o];
+            sa[i] = sa[i + o];
         }
-        sv[i] = a;
-        sn[i] = n;
-        sj[i] = n * mej;
-        sm[i] = n * cm;
+        __syncthreads();
+    }
+    if (sv[0] == -INFINITY) {  // no samples: the whole CTA
+        if (i == 0) out.ln[slot] = -INFINITY;
+        return;
+    }
+    const int ref = e0 + sa[0];
+    const double r = (double)(e0 + i - ref);
+    double v = 0.0, vn = 0.0, mej = 0.0, cm = 0.0;
+    __syncthreads();
+    if (n > 0.0) {
+        // near the heaviest bin these are differences of near numbers
+        v = exp(-(p.slope * r) - (s.lw[e0 + i] - s.lw[ref]));
+        vn = v * n;
+        mej = s.mej[e0 + i] - s.mej[ref];
+        cm = s.cm[e0 + i] - s.cm[ref];
+    }
+    if (i < 64) {
+        sv[i] = vn;
+        sj[i] = vn * mej;
+        sm[i] = vn * cm;
     }
     __syncthreads();
     for (int o = 32; o > 0; o >>= 1) {
         if (i < o) {
-            sn[i] += sn[i + o];
+            sv[i] += sv[i + o];
             sj[i] += sj[i + o];
             sm[i] += sm[i + o];
-            sv[i] = fmax(sv[i], sv[i + o]);
         }
         __syncthreads();
     }
-    // the references: the means
-    const double mj = sn[0] > 0.0 ? sj[0] / sn[0] : 0.0, mm = sn[0] > 0.0 ? sm[0] / sn[0] : 0.0;
-    const double vb = sn[0] > 0.0 ? sv[0] : 0.0;
+    const double mj = s.mej[ref] + sj[0] / sv[0], mm = s.cm[ref] + sm[0] / sv[0];
     if (i == 0) {
-        out.v[slot] = vb;
+        out.ln[slot] = log(s.n[ref]);
         out.E[slot] = e_min + ref;
-        out.lw[slot] = lref;
+        out.mid[slot] = mid - ref;
+        out.lw[slot] = s.lw[ref];
         out.mj[slot] = mj;
         out.mm[slot] = mm;
-        out.used[slot] = sn[0] > 0.0;
     }
     if (i < p.B) {
-        const double rho = (double)r * (2.0 / p.B);  // exact: B is a power of 2
-        const double v = n > 0.0 ? exp(a - vb) : 0.0;
-        const double vn = v * n, dj = mej - mj, dm = cm - mm;
+        const double rho = (double)(e0 + i - mid) * (2.0 / p.B);  // exact: B is a power of 2
+        const double dj = n > 0.0 ? s.mej[e0 + i] - mj : 0.0, dm = n > 0.0 ? s.cm[e0 + i] - mm : 0.0;
         f[0][i] = vn;
-        f[1][i] = vn * (double)r;
+        f[1][i] = vn * r;
         f[2][i] = vn * dj;
         f[3][i] = vn * dm;
         f[4][i] = n > 0.0 ? v * s.q2[e0 + i] : 0.0;
         f[5][i] = n > 0.0 ? v * s.q4[e0 + i] : 0.0;
-        f[6][i] = vn * (dj * (double)r);
+        f[6][i] = vn * (dj * r);
         f[7][i] = n > 0.0 ? v * s.vb[e0 + i] + vn * (dm * dm) : 0.0;
         double pw = 1.0;
         t[0][i] = 1.0;
@@ -942,11 +966,11 @@ block_coef_kernel(BinStats<double> s, int nE, int e_min, BlockPlan p, Blocks out
     }
 }
 
-// ln A for one field, relative to the reference block's (E0, l0): the product
-// and the difference without rounding, their sum rounded once.
-__device__ __forceinline__ double block_exponent(double c, int dE, double lw, double l0)
+// -c e - (lw - l0), e the distance from the reference bin: the product and the
+// difference without rounding, their sum rounded once.
+__device__ __forceinline__ double block_exponent(double c, double e, double lw, double l0)
 {
-    const double e = (double)dE, p = __dmul_rn(c, e), pe = fma(c, e, -p);
+    const double p = __dmul_rn(c, e), pe = fma(c, e, -p);
     const double l = __dsub_rn(lw, l0), bb = __dsub_rn(l, lw);
     const double le = __dsub_rn(__dsub_rn(lw, __dsub_rn(l, bb)), __dadd_rn(l0, bb));
     return (-p - l) - (pe + le);
@@ -983,22 +1007,23 @@ block_grid_kernel(Blocks bl, BlockPlan p, double beta, int V, const double *__re
 {
     __shared__ double shv[32];
     __shared__ int she[32];
-    __shared__ double sh[kRgThreads / 32 * 6];
+    __shared__ double sh[kRgThreads / 32 * kStats];
     const int t = threadIdx.x, k0 = blockIdx.x * KK;
     const size_t slots = (size_t)p.per * kRgThreads;
-    double c[KK], x[KK], l0[KK], v0[KK], J0[KK], M0[KK];
+    double c[KK], x[KK], u[KK], l0[KK], J0[KK], M0[KK];
     int E0[KK];
-    // the reference of each field: its block of the largest A
+    // the reference of each field: its heaviest block
 #pragma unroll
     for (int k = 0; k < KK; ++k) {
         c[k] = cgrid[min(k0 + k, n_grid - 1)];
-        x[k] = -(c[k] - p.slope) * (0.5 * p.B);
+        u[k] = -(c[k] - p.slope);
+        x[k] = u[k] * (0.5 * p.B);
         double best = -INFINITY;
         int at = 0x7FFFFFFF;
         for (int i = 0; i < p.per; ++i) {
             const int q = i * kRgThreads + t;
-            if (t * p.per + i < p.nblk && bl.used[q]) {
-                const double a = (-(c[k] * (double)bl.E[q]) - bl.lw[q]) + bl.v[q];
+            if (t * p.per + i < p.nblk && bl.ln[q] > -INFINITY) {
+                const double a = (-(c[k] * (double)bl.E[q]) - bl.lw[q]) + bl.ln[q];
                 if (a > best) {
                     best = a;
                     at = q;
@@ -1006,40 +1031,30 @@ block_grid_kernel(Blocks bl, BlockPlan p, double beta, int V, const double *__re
             }
         }
         block_argmax(best, at, shv, she);
-        if (at >= (int)slots) at = 0;  // no sample lies in the window (the call fails)
-        E0[k] = bl.E[at];
-        l0[k] = bl.lw[at];
-        v0[k] = bl.v[at];
-        J0[k] = bl.mj[at];
-        M0[k] = bl.mm[at];
+        const bool none = at >= (int)slots;  // no sample lies in the window (the call fails)
+        E0[k] = none ? 0 : bl.E[at];
+        l0[k] = none ? 0.0 : bl.lw[at];
+        J0[k] = none ? 0.0 : bl.mj[at];
+        M0[k] = none ? 0.0 : bl.mm[at];
     }
     double S[KK][kStats];
 #pragma unroll
     for (int k = 0; k < KK; ++k)
 #pragma unroll
         for (int j = 0; j < kStats; ++j) S[k][j] = 0.0;
-    // references of this thread's sums: those of its first block that counts
-    bool have = false;
-    int Et = 0;
-    double Jt = 0.0, Mt = 0.0;
     for (int i = 0; i < p.per; ++i) {
         const int q = i * kRgThreads + t;
-        if (t * p.per + i >= p.nblk || !bl.used[q]) continue;
+        if (t * p.per + i >= p.nblk || bl.ln[q] == -INFINITY) continue;
         const int Eb = bl.E[q];
+        const double lb = bl.lw[q], mid = (double)bl.mid[q];
         double A[KK];
         bool any = false;
 #pragma unroll
         for (int k = 0; k < KK; ++k) {
-            A[k] = exp(block_exponent(c[k], Eb - E0[k], bl.lw[q], l0[k]) + (bl.v[q] - v0[k]));
+            A[k] = exp(fma(u[k], mid, block_exponent(c[k], (double)(Eb - E0[k]), lb, l0[k])));
             any = any || A[k] > 0.0;
         }
         if (!any) continue;
-        if (!have) {
-            have = true;
-            Et = Eb;
-            Jt = bl.mj[q];
-            Mt = bl.mm[q];
-        }
         double a[kStats][KK];
 #pragma unroll
         for (int j = 0; j < kStats; ++j) {
@@ -1053,9 +1068,10 @@ block_grid_kernel(Blocks bl, BlockPlan p, double beta, int V, const double *__re
                 for (int k = 0; k < KK; ++k) a[j][k] = fma(a[j][k], x[k], cg);
             }
         }
-        const double dE = (double)(Eb - Et), dJ = bl.mj[q] - Jt, dM = bl.mm[q] - Mt;
+        const double Jb = bl.mj[q], Mb = bl.mm[q];
 #pragma unroll
         for (int k = 0; k < KK; ++k) {
+            const double dE = (double)(Eb - E0[k]), dJ = Jb - J0[k], dM = Mb - M0[k];
             const double n0 = A[k] * a[0][k], e1 = A[k] * a[1][k], j1 = A[k] * a[2][k], m1 = A[k] * a[3][k];
             const double e2 = fma(n0, dE, e1), j2 = fma(n0, dJ, j1);
             S[k][0] += n0;
@@ -1064,30 +1080,24 @@ block_grid_kernel(Blocks bl, BlockPlan p, double beta, int V, const double *__re
             S[k][3] += fma(n0, dM, m1);
             S[k][4] += A[k] * a[4][k];
             S[k][5] += A[k] * a[5][k];
-            // sum n (J - Jt)(E - Et) and sum (vb + n (m - Mt)^2)
+            // sum n (J - J0)(E - E0) and sum (vb + n (m - M0)^2)
             S[k][6] += fma(A[k], a[6][k], fma(j1, dE, e2 * dJ));
             S[k][7] += fma(A[k], a[7][k], dM * fma(n0, dM, m1 + m1));
         }
     }
 #pragma unroll
     for (int k = 0; k < KK; ++k) {
-        const double *R = S[k];
-        // the means relative to the reference block's
-        double T[6] = {R[0], fma(R[0], (double)(Et - E0[k]), R[1]), fma(R[0], Jt - J0[k], R[2]),
-                  fma(R[0], Mt - M0[k], R[3]), R[4], R[5]};
-        block_sum_plain<6>(T, sh);
+        double (&T)[kStats] = S[k];
+        block_sum_plain<kStats>(T, sh);
+        // the means relative to the reference, and the sums about them
         const double Z = T[0], mE = T[1] / Z, mJ = T[2] / Z, mu = T[3] / Z;
-        const double dE = (double)(Et - E0[k]) - mE, dJ = (Jt - J0[k]) - mJ, dM = (Mt - M0[k]) - mu;
-        double U[2] = {R[6] + dE * R[2] + dJ * R[1] + dE * dJ * R[0],
-                  R[7] + 2.0 * dM * R[3] + dM * dM * R[0]};
-        block_sum_plain<2>(U, sh);
         if (t == 0 && k0 + k < n_grid) {
             double *o = out + 5 * (int64_t)(k0 + k);
             const double m2 = T[4] / Z, m4 = T[5] / Z;
             o[0] = J0[k] + mJ;
             o[1] = (double)E0[k] + mE;
-            o[2] = -beta * (U[0] / Z);
-            o[3] = beta * (double)V * (U[1] / Z);
+            o[2] = -beta * (T[6] / Z - mE * mJ);
+            o[3] = beta * (double)V * (T[7] / Z - mu * mu);
             o[4] = 1.0 - m4 / (3.0 * m2 * m2);
         }
     }

@@ -264,3 +264,33 @@ def test_fp64_blocks_of_bins_every_size():
             ref = oracle.reweight(ej, ed, m, lnW, 0, beta, n_e - 1, grid)
             got = muca().reweight(dev(ej), dev(ed), dev(m), lnW, 0, beta, n_e - 1, grid, 64)
             assert (rel_err(got, ref) <= TOL[64]).all(), (width, rel_err(got, ref).max(axis=0))
+
+
+@pytest.mark.parametrize("bd", [-25.0, -18.0, -10.0, 10.0, 18.0, 25.0])
+def test_fp64_pinned_distributions(bd):
+    """Fields so far from the transition that the distribution sits on the last
+    bins of one end of E_Delta (weights -ln of the binomial density of states;
+    at low temperature the same happens next to the transition): C and chi
+    against binary128, point by point, for a single field, narrow, wider and
+    wide grids, and enough unordered fields that several share a block.
+
+    Per point, no curve's scale: the means of E_J are below 1536 and rounded to
+    1.1e-13, their differences between neighbouring bins at least 1, so C holds
+    to a few 1e-13."""
+    rng = np.random.default_rng(5)
+    V, beta = 512, 0.8
+    n = rng.integers(40, 120, V + 1)
+    ed = np.repeat(np.arange(V + 1), n)
+    ej = -3 * ed + rng.integers(-3, 4, ed.size)
+    m = np.clip(np.rint(0.7 * ed).astype(int) + rng.integers(-30, 31, ed.size), -ed, ed)
+    lf = np.concatenate([[0.0], np.cumsum(np.log(np.arange(1, V + 1)))])
+    e = np.arange(V + 1)
+    lnW = -(lf[V] - lf - lf[::-1] + e * np.log(2.0))
+    many = bd + 0.03 * np.linspace(-1, 1, 701)[rng.permutation(701)]
+    for grid, ks in [(np.array([bd]), [0]), (bd + np.array([-0.03, 0.01, 0.03]), [0, 1, 2]),
+                     (bd + np.array([0.25, -0.25, 0.1]), [0, 1, 2]),
+                     (np.array([bd, -25.0, 25.0, 3.0]), [0, 1, 2, 3]), (many, [0, 333, 700])]:
+        ref = oracle.reweight_q(ej, ed, m, lnW, 0, beta, V, grid[ks] / beta)
+        got = muca().reweight(dev(ej), dev(ed), dev(m), lnW, 0, beta, V, grid / beta, 64)[ks]
+        err = np.abs(got - ref) / np.abs(ref)
+        assert (err[:, :4] <= TOL[64]).all(), (grid[:4], err.max(axis=0))
