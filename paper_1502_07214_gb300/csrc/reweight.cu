@@ -757,7 +757,92 @@ grid_kernel_f32(BinStats<float> s, int nE, int e_min, float beta, int V,
     }
 }
 
-// ------------------------------------------------------------ FP64 stage B
+// ------------------------------------------- FP64 stage B, bin by bin
+// Grids that are too wide for blocks of bins (below): every field visits every
+// occupied bin, the sums are compensated, C and chi are taken in a second pass
+// about the means.
+// Exponent of Eq. 3: a = -(c E) - lnW(E), c = beta Delta_k.  It is used to
+// find the bin E* of the largest weight; the normalised exponents are then
+// formed as -c (E - E*) - (lnW(E) - lnW(E*)) so that two O(beta Delta V) numbers
+// are never subtracted.
+__device__ __forceinline__ double expo64(double c, int E, double lw)
+{
+    return __dsub_rn(-__dmul_rn(c, (double)E), lw);
+}
+
+__device__ __forceinline__ double rel64(double c, int dE, double lw, double lstar)
+{
+    return __dsub_rn(-__dmul_rn(c, (double)dE), __dsub_rn(lw, lstar));
+}
+
+__global__ void __launch_bounds__(256)
+grid_kernel_f64(BinStats<double> s, int nE, int e_min, double beta, int V,
+                const double *__restrict__ cgrid, double *__restrict__ out)
+{
+    __shared__ double sh[64];
+    __shared__ int she[32];
+    const int k = blockIdx.x;
+    const double c = cgrid[k];
+    double amax = -INFINITY;
+    int estar = 0x7FFFFFFF;
+    for (int e = threadIdx.x; e < nE; e += blockDim.x)
+        if (s.n[e] > 0) {
+            const double a = expo64(c, e_min + e, s.lw[e]);
+            if (a > amax) {
+                amax = a;
+                estar = e;
+            }
+        }
+    block_argmax(amax, estar, sh, she);
+    const double lstar = s.lw[estar];
+    KSum<double> acc[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) acc[i].init();
+    for (int e = threadIdx.x; e < nE; e += blockDim.x) {
+        const double n = s.n[e];
+        if (n <= 0) continue;
+        const double d = rel64(c, e - estar, s.lw[e], lstar);
+        if (d < -800.0) continue;
+        const double w = exp(d);
+        const double wn = w * n;
+        acc[0].add(wn);
+        acc[1].add(wn * (double)(e_min + e));
+        acc[2].add(wn * s.mej[e]);
+        acc[3].add(wn * s.cm[e]);
+        acc[4].add(w * s.q2[e]);
+        acc[5].add(w * s.q4[e]);
+    }
+    double S[6];
+    block_sum<double, 6>(acc, S, sh);
+    const double Z = S[0], mE = S[1] / Z, mJ = S[2] / Z, mu = S[3] / Z;
+    KSum<double> acc2[2];
+    acc2[0].init();
+    acc2[1].init();
+    for (int e = threadIdx.x; e < nE; e += blockDim.x) {
+        const double n = s.n[e];
+        if (n <= 0) continue;
+        const double d = rel64(c, e - estar, s.lw[e], lstar);
+        if (d < -800.0) continue;
+        const double w = exp(d);
+        const double wn = w * n;
+        acc2[0].add(wn * ((s.mej[e] - mJ) * ((double)(e_min + e) - mE)));
+        const double dm = s.cm[e] - mu;
+        acc2[1].add(w * s.vb[e] + wn * (dm * dm));
+    }
+    double S2[2];
+    block_sum<double, 2>(acc2, S2, sh);
+    if (threadIdx.x == 0) {
+        double *o = out + 5 * (int64_t)k;
+        o[0] = mJ;
+        o[1] = mE;
+        o[2] = -beta * (S2[0] / Z);
+        o[3] = beta * (double)V * (S2[1] / Z);
+        const double m2 = S[4] / Z, m4 = S[5] / Z;
+        o[4] = 1.0 - m4 / (3.0 * m2 * m2);
+    }
+}
+
+// ------------------------------------------- FP64 stage B, blocks of bins
 // The weight of Eq. 3 factorises over a block of B consecutive bins: with
 // E_b the block's heaviest bin (the largest n exp(-s E - lnW), s a slope common
 // to the grid) and r = E - E_b,
@@ -802,8 +887,12 @@ struct BlockPlan {
 // Block size and degree for fields c in [lo, hi].  |x| <= 1.2 keeps the
 // polynomial's alternating terms within e^2.4 of their sum.  The degree is the
 // first whose remainder |x|^(deg+1) / (deg+1)! is below a sixteenth of the
-// rounding.  A grid too wide for blocks of 8 takes single bins (degree 0): 20
-// coefficients per sum and block would outgrow the bins below that.
+// rounding.  B = 0: the grid is too wide for blocks of 8, its fields go bin by
+// bin (8 sums of 20 coefficients cost as much as 8 bins there).  Measured at
+// beta = 0.7, 4096 fields, 6.4e5 samples: half width 0.42 (blocks of 8) 5.4 ms
+// for 32769 bins and 40.5 ms for 262145 against 11.3 and 45.5 bin by bin; half
+// width 1 and 20 (bin by bin) 8.9 and 6.3 ms for 32769 bins, where blocks of
+// one bin took 15.1 and 13.4.
 BlockPlan block_plan(double lo, double hi, int nE)
 {
     BlockPlan p{};
@@ -811,7 +900,7 @@ BlockPlan block_plan(double lo, double hi, int nE)
     const double w = 0.5 * (hi - lo);
     for (int B = 64; B >= 8 && !p.B; B /= 2)
         if (w * (B / 2) <= kXMax) p.B = B;
-    if (!p.B) p.B = 1;
+    if (!p.B) return p;
     const double x = w * (p.B / 2), eps = 0x1p-57;
     double term = 1.0;
     for (p.deg = 0; p.deg < kDegMax; ++p.deg) {
@@ -853,7 +942,7 @@ struct Blocks {
 
 size_t block_bytes(const BlockPlan &p)
 {
-    const size_t slots = (size_t)p.per * kRgThreads;
+    const size_t slots = (size_t)p.per * kRgThreads;  // 0 without blocks
     return slots * ((kStats * (p.deg + 1) + 4) * sizeof(double) + 2 * sizeof(int));
 }
 
@@ -1265,8 +1354,10 @@ int reweight_on_scratch(const int32_t *e_j, const int32_t *e_d, const int32_t *m
                             cudaMemcpyHostToDevice, st));
         stats_kernel_f64<<<sb, 256, 0, st>>>(b, n_e, V, d_lnW, s);
         RCK(cudaGetLastError());
-        if (n_grid > 0)
+        if (n_grid > 0 && plan.B)
             RCK(launch_blocks(s, n_e, e_min, beta, V, plan, blocks, d_c, n_grid, d_out, nsm, st));
+        else if (n_grid > 0)
+            grid_kernel_f64<<<n_grid, 256, 0, st>>>(s, n_e, e_min, beta, V, d_c, d_out);
         RCK(cudaGetLastError());
     } else {
         BinStats<float> s;
