@@ -89,25 +89,30 @@ constexpr int kPkThreads = 256;
 
 // ------------------------------------------------------------- blocks of bins
 // The bisection evaluates the same sums at some sixty fields of a narrow
-// interval.  Over a block of B consecutive bins the weight factorises: with
-// r = E - E_b, s the interval's middle field beta Delta, and v_b the block's
-// largest exponent at s,
-//   exp(-c E - lnW(E)) = exp(a_b - (c - s) (E_b - E_r)) exp(-(c - s) r) V(E),
-//   a_b = -s (E_b - E_r) - (lnW(E_b) - lnW(E_r)) + v_b,
-//   V = exp(-s r - (lnW(E) - lnW(E_b)) - v_b) <= 1,
+// interval.  Over a block of B consecutive bins the weight factorises: with s
+// the interval's middle field beta Delta, E_b the block's heaviest bin (the
+// largest n exp(-s E - lnW)), E_mid its middle and r = E - E_b,
+//   exp(-c E - lnW(E)) = exp(a_b - (c - s) (E_mid - E_r)) exp(-(c - s) (E - E_mid)) V(E),
+//   a_b = -s (E_b - E_r) - (lnW(E_b) - lnW(E_r)),   V = exp(-s r - (lnW(E) - lnW(E_b))),
 // and |c - s| B / 2 is small in the whole interval, so the middle factor is its
 // Taylor polynomial in x = -(c - s) B / 2 and each weighted sum over the block
 // is a polynomial in x, its coefficients formed once per call.  A step then
 // takes one exponential and 6 deg multiply-adds per block, where the bins took
 // an exponential and some hundred FP64 instructions each (FP64 runs at two
-// multiply-adds per clock and SM).  Sums are taken about references near the
-// bins and moved to the common mean at the end of the step.
+// multiply-adds per clock and SM).
+// Sums are taken about bins that hold weight (inside a block its heaviest bin
+// and weighted mean E_J, then the heaviest block's of the CTA) and moved to the
+// common mean at the end of the step.  a_b is kept as a pair (its magnitude
+// is that of beta Delta V, the differences between blocks that count are
+// small).  C* of a series that fills 61 of 262145 bins, against binary128:
+// 1e-15, as with compensated sums over the bins; with a_b rounded once 8e-13.
 // Measured: 21 data sets of 4.1e7 samples, 32769 bins, 60 steps: the bisection
-// kernel took 8.7 ms bin by bin, now 0.75 ms.
+// kernel took 8.7 ms bin by bin, now 0.73 ms.
 constexpr int kPkStats = 6;    // n, n r, n r^2, n J, n J r, n J r^2 (J about the block's mean)
 constexpr int kPkDegMax = 20;
 constexpr int kPkMaxB = 512;
 constexpr int kPkStepThreads = 64;
+constexpr int kPkMaxCta = 8;   // CTAs per cluster
 
 struct PkPlan {
     int B, nblk, deg, ncta, per, slots;  // slots = ncta kPkStepThreads per
@@ -143,17 +148,18 @@ __host__ __device__ inline int pk_slot(const PkPlan &p, int b)
     return (b % p.per) * (p.ncta * kPkStepThreads) + b / p.per;
 }
 
-// Per set and slot: coefficients [deg + 1][kPkStats], a_b, the block's mean E_J,
-// whether it has samples.
+// Per set and slot: coefficients [deg + 1][kPkStats], a_b = ah + al, the
+// block's weighted mean E_J, ln of the samples in its heaviest bin (-inf for a
+// block without samples), that bin (relative to e_min).
 struct PkBlocks {
-    double *coef, *a, *mj;
-    int *used;
+    double *coef, *ah, *al, *mj, *ln;
+    int *E;
 };
 
 size_t pk_block_bytes(const PkPlan &p, int n_sets)
 {
     return (size_t)n_sets * p.slots *
-           ((kPkStats * (p.deg + 1) + 2) * sizeof(double) + sizeof(int));
+           ((kPkStats * (p.deg + 1) + 4) * sizeof(double) + sizeof(int));
 }
 
 PkBlocks pk_block_layout(const PkPlan &p, int n_sets, char *mem)
@@ -161,9 +167,11 @@ PkBlocks pk_block_layout(const PkPlan &p, int n_sets, char *mem)
     const size_t n = (size_t)n_sets * p.slots;
     PkBlocks b;
     b.coef = (double *)mem;
-    b.a = b.coef + n * kPkStats * (p.deg + 1);
-    b.mj = b.a + n;
-    b.used = (int *)(b.mj + n);
+    b.ah = b.coef + n * kPkStats * (p.deg + 1);
+    b.al = b.ah + n;
+    b.mj = b.al + n;
+    b.ln = b.mj + n;
+    b.E = (int *)(b.ln + n);
     return b;
 }
 
@@ -171,8 +179,8 @@ __constant__ double pk_inv[kPkDegMax + 1] = {
     0.0, 1.0, 1.0 / 2, 1.0 / 3, 1.0 / 4, 1.0 / 5, 1.0 / 6, 1.0 / 7, 1.0 / 8, 1.0 / 9, 1.0 / 10,
     1.0 / 11, 1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17, 1.0 / 18, 1.0 / 19, 1.0 / 20};
 
-// Reference bin of block b (relative to e_min): its middle.
-__device__ __forceinline__ int pk_ref(const PkPlan &p, int b, int nE)
+// Middle bin of block b (relative to e_min).
+__device__ __forceinline__ int pk_mid(const PkPlan &p, int b, int nE)
 {
     return min(b * p.B + p.B / 2, nE - 1);
 }
@@ -182,47 +190,85 @@ __global__ void __launch_bounds__(128)
 pk_coef_kernel(const double *__restrict__ n_all, const double *__restrict__ mj_all,
                const double *__restrict__ lnW, int nE, PkPlan p, PkBlocks out)
 {
-    __shared__ double f[kPkStats][64], t[kPkDegMax + 1][64];
-    __shared__ double red[3][4];
+    __shared__ double f[kPkStats][64], t[kPkDegMax + 1][64], sv[kPkMaxB];
+    __shared__ double red[2][4];
+    __shared__ int ired[4];
     const int b = blockIdx.x, d = blockIdx.y, i = threadIdx.x, lane = i & 31, wid = i >> 5;
     const double *n = n_all + (size_t)d * nE, *mj = mj_all + (size_t)d * nE;
-    const int e0 = b * p.B, e1 = min(e0 + p.B, nE), ref = pk_ref(p, b, nE);
-    const double lref = lnW[ref];
-    auto expo = [&](int e) { return -(p.slope * (double)(e - ref)) - (lnW[e] - lref); };
-    double vb = -INFINITY, sn = 0.0, sj = 0.0;
+    const int e0 = b * p.B, e1 = min(e0 + p.B, nE), mid = pk_mid(p, b, nE);
+    const size_t slot = (size_t)d * p.slots + pk_slot(p, b), stride = (size_t)gridDim.y * p.slots;
+    // the heaviest bin (to the precision of an FP32 logarithm: any bin near it serves)
+    double best = -INFINITY;
+    int ref = -1;
     for (int e = e0 + i; e < e1; e += 128)
         if (n[e] > 0.0) {
-            vb = fmax(vb, expo(e));
-            sn += n[e];
-            sj += n[e] * mj[e];
+            const double v = (-(p.slope * (double)(e - mid)) - (lnW[e] - lnW[mid])) +
+                             (double)__logf((float)n[e]);
+            if (ref < 0 || v > best) {
+                best = v;
+                ref = e;
+            }
         }
     for (int o = 16; o > 0; o >>= 1) {
-        vb = fmax(vb, __shfl_xor_sync(0xFFFFFFFFu, vb, o));
+        const double v2 = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+        const int r2 = __shfl_xor_sync(0xFFFFFFFFu, ref, o);
+        if (r2 >= 0 && (ref < 0 || v2 > best || (v2 == best && r2 < ref))) {
+            best = v2;
+            ref = r2;
+        }
+    }
+    if (lane == 0) {
+        red[0][wid] = best;
+        ired[wid] = ref;
+    }
+    __syncthreads();
+    best = red[0][0];
+    ref = ired[0];
+    for (int k = 1; k < 4; ++k)
+        if (ired[k] >= 0 && (ref < 0 || red[0][k] > best)) {
+            best = red[0][k];
+            ref = ired[k];
+        }
+    if (ref < 0) {  // no samples: the whole CTA
+        if (i == 0) out.ln[slot] = -INFINITY;
+        return;
+    }
+    __syncthreads();
+    const double lref = lnW[ref], jref = mj[ref];
+    double sn = 0.0, sj = 0.0;
+    for (int e = e0 + i; e < e1; e += 128) {
+        // near the heaviest bin the exponents are differences of near numbers
+        const double vn = n[e] > 0.0 ? exp(-(p.slope * (double)(e - ref)) - (lnW[e] - lref)) * n[e] : 0.0;
+        sv[e - e0] = vn;
+        sn += vn;
+        sj += n[e] > 0.0 ? vn * (mj[e] - jref) : 0.0;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
         sn += __shfl_xor_sync(0xFFFFFFFFu, sn, o);
         sj += __shfl_xor_sync(0xFFFFFFFFu, sj, o);
     }
     if (lane == 0) {
-        red[0][wid] = vb;
-        red[1][wid] = sn;
-        red[2][wid] = sj;
+        red[0][wid] = sn;
+        red[1][wid] = sj;
     }
     __syncthreads();
-    vb = fmax(fmax(red[0][0], red[0][1]), fmax(red[0][2], red[0][3]));
-    sn = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
-    sj = (red[2][0] + red[2][1]) + (red[2][2] + red[2][3]);
-    const double jb = sn > 0.0 ? sj / sn : 0.0;
-    const size_t slot = (size_t)d * p.slots + pk_slot(p, b), stride = (size_t)gridDim.y * p.slots;
+    sn = (red[0][0] + red[0][1]) + (red[0][2] + red[0][3]);
+    sj = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
+    const double jb = jref + sj / sn;
     if (i == 0) {
-        // a_b: the product and the difference without rounding
+        // a_b: the product and the differences without rounding, as a pair
         const int er = nE / 2;
-        const double x = (double)(ref - er), pr = __dmul_rn(p.slope, x), pe = fma(p.slope, x, -pr);
+        const double x = (double)(ref - er), a1 = -__dmul_rn(p.slope, x), pe = fma(p.slope, x, a1);
         const double l0 = lnW[er], l = __dsub_rn(lref, l0), bb = __dsub_rn(l, lref);
         const double le = __dsub_rn(__dsub_rn(lref, __dsub_rn(l, bb)), __dadd_rn(l0, bb));
-        out.a[slot] = sn > 0.0 ? ((-pr - l) - (pe + le)) + vb : 0.0;
+        const double h = __dsub_rn(a1, l), u = __dsub_rn(h, a1);
+        const double he = __dsub_rn(__dsub_rn(a1, __dsub_rn(h, u)), __dadd_rn(l, u));
+        out.ah[slot] = h;
+        out.al[slot] = he - (pe + le);
         out.mj[slot] = jb;
-        out.used[slot] = sn > 0.0;
+        out.ln[slot] = log(n[ref]);
+        out.E[slot] = ref;
     }
-    if (!(sn > 0.0)) return;  // the whole CTA
     double c[2] = {0.0, 0.0};  // this thread's coefficients i and i + 128
     for (int k0 = e0; k0 < e1; k0 += 64) {
         __syncthreads();
@@ -230,14 +276,14 @@ pk_coef_kernel(const double *__restrict__ n_all, const double *__restrict__ mj_a
             const int e = k0 + i;
             const bool in = e < e1 && n[e] > 0.0;
             const double r = (double)(e - ref), dj = in ? mj[e] - jb : 0.0;
-            const double vn = in ? exp(expo(e) - vb) * n[e] : 0.0;
+            const double vn = in ? sv[e - e0] : 0.0;
             f[0][i] = vn;
             f[1][i] = vn * r;
             f[2][i] = vn * (r * r);
             f[3][i] = vn * dj;
             f[4][i] = vn * (dj * r);
             f[5][i] = vn * (dj * r * r);
-            const double rho = r * (2.0 / p.B);  // exact: B is a power of 2
+            const double rho = (double)(e - mid) * (2.0 / p.B);  // exact: B is a power of 2
             double pw = 1.0;
             t[0][i] = 1.0;
             for (int q = 1; q <= p.deg; ++q) {
@@ -261,11 +307,17 @@ pk_coef_kernel(const double *__restrict__ n_all, const double *__restrict__ mj_a
     }
 }
 
-// One CTA's part of a step, read by every CTA of the cluster: its sums relative
-// to the largest exponent mx, about (E, J).
+// A block as the reference of a CTA's sums (E < 0: none).
+struct PkRef {
+    double ah, al, ln, J;
+    int mid, E;
+};
+
+// One CTA's part of a step: its sums R relative to the exponent of its reference
+// block, about (E, J) of that block, then the block's ah, al, ln, J, (E, mid).
+constexpr int kPkWords = kPkStats + 5;
 struct PkPart {
-    double mx, J, R[kPkStats];
-    int E;
+    double w[kPkWords];
 };
 
 // Move the sums R of n, n E, n E^2, n J, n J E, n J E^2 to references that lie
@@ -283,14 +335,15 @@ __device__ __forceinline__ void pk_shift(double (&R)[kPkStats], double dE, doubl
 
 // Covariance <(E_J - <E_J>)(E_Delta - <E_Delta>)> and third moment
 // <(E_J - <E_J>)(E_Delta - <E_Delta>)^2> of data set d at field c = beta Delta.
-// The cluster's CTAs combine their parts through slot `slot` (slots alternate,
-// so one cluster barrier per step suffices); every thread gets the result.
-// mx, at: the largest exponent of the CTA's blocks and its block, found anew
-// when `find` is set, else kept as a fixed reference.
+// The CTAs hand their parts to one another in slot `slot` of each one's `part`
+// (slots alternate, so one cluster barrier per step suffices); every thread gets
+// the result.
+// ref: the heaviest of the CTA's blocks, found anew when `find` is set, else kept
+// as a fixed reference.
 // Results: the moments times z = sum n (the sign of the third is all that a
 // step needs).
 __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const PkBlocks &bl,
-                           const PkPlan &p, int d, int nE, double c, bool find, double &mx, int &at,
+                           const PkPlan &p, int d, int nE, double c, bool find, PkRef &ref,
                            double *sh, int *shi, double &cov, double &third, double &z0)
 {
     const int q = (int)cl.block_rank(), t = (int)threadIdx.x, lane = t & 31, wid = t >> 5;
@@ -298,15 +351,14 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
     const size_t base = (size_t)d * p.slots, stride = (size_t)(gridDim.x / p.ncta) * p.slots;
     const double dc = c - p.slope, x = -dc * (0.5 * p.B);
     const int er = nE / 2;
-    // the CTA's largest exponent and its block
     if (find) {
-        mx = -INFINITY;
-        at = -1;
+        double mx = -INFINITY;
+        int at = -1;
         for (int i = 0; i < p.per; ++i) {
             const int b = g * p.per + i;
             const size_t k = base + (size_t)i * gs + g;
-            if (b >= p.nblk || !bl.used[k]) continue;
-            const double v = fma(-dc, (double)(pk_ref(p, b, nE) - er), bl.a[k]);
+            if (b >= p.nblk || bl.ln[k] == -INFINITY) continue;
+            const double v = fma(-dc, (double)(pk_mid(p, b, nE) - er), bl.ah[k]) + bl.ln[k];
             if (v > mx) {
                 mx = v;
                 at = b;
@@ -331,18 +383,23 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
                 mx = sh[i];
                 at = shi[i];
             }
+        ref = PkRef{0.0, 0.0, -INFINITY, 0.0, er, -1};
+        if (at >= 0) {
+            const size_t k = base + pk_slot(p, at);
+            ref = PkRef{bl.ah[k], bl.al[k], bl.ln[k], bl.mj[k], pk_mid(p, at, nE), bl.E[k]};
+        }
     }
-    const int Ec = at >= 0 ? pk_ref(p, at, nE) : er;
-    const double Jc = at >= 0 ? bl.mj[base + pk_slot(p, at)] : 0.0;
     double S[kPkStats];
 #pragma unroll
     for (int j = 0; j < kPkStats; ++j) S[j] = 0.0;
     for (int i = 0; i < p.per; ++i) {
         const int b = g * p.per + i;
         const size_t k = base + (size_t)i * gs + g;
-        if (b >= p.nblk || !bl.used[k]) continue;
-        const int E = pk_ref(p, b, nE);
-        const double A = exp(fma(-dc, (double)(E - er), bl.a[k]) - mx);
+        // loaded together (slots past the last block are allocated, and not used)
+        const double ln = bl.ln[k], ah = bl.ah[k], al = bl.al[k], mj = bl.mj[k];
+        const int E = bl.E[k];
+        if (b >= p.nblk || ln == -INFINITY) continue;
+        const double A = exp(fma(-dc, (double)(pk_mid(p, b, nE) - ref.mid), (ah - ref.ah) + (al - ref.al)));
         if (!(A > 0.0)) continue;
         double R[kPkStats];
 #pragma unroll
@@ -351,7 +408,7 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
 #pragma unroll
             for (int j = 0; j < kPkStats; ++j)
                 R[j] = fma(R[j], x, bl.coef[(size_t)(u * kPkStats + j) * stride + k]);
-        pk_shift(R, (double)(E - Ec), bl.mj[k] - Jc);
+        pk_shift(R, (double)(E - ref.E), mj - ref.J);
 #pragma unroll
         for (int j = 0; j < kPkStats; ++j) S[j] = fma(A, R[j], S[j]);
     }
@@ -363,42 +420,56 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
 #pragma unroll
         for (int j = 0; j < kPkStats; ++j) sh[wid * kPkStats + j] = S[j];
     __syncthreads();
-    if (t == 0) {
-        PkPart &m = part[slot];
-        m.mx = mx;
-        m.E = Ec;
-        m.J = Jc;
-#pragma unroll
-        for (int j = 0; j < kPkStats; ++j) {
-            double v = sh[j];
-            for (int i = 1; i < kPkStepThreads / 32; ++i) v += sh[i * kPkStats + j];
-            m.R[j] = v;
-        }
+    // this CTA's part to every CTA of the cluster, a word per thread (reading the
+    // others' parts instead waits for distributed shared memory once more)
+    for (int i = t; i < kPkWords * p.ncta; i += kPkStepThreads) {
+        const int r = i / kPkWords, w = i - r * kPkWords;
+        double v = 0.0;
+        if (w < kPkStats)
+            for (int k = 0; k < kPkStepThreads / 32; ++k) v += sh[k * kPkStats + w];
+        else
+            v = w == kPkStats       ? ref.ah
+                : w == kPkStats + 1 ? ref.al
+                : w == kPkStats + 2 ? ref.ln
+                : w == kPkStats + 3 ? ref.J
+                                    : __hiloint2double(ref.E, ref.mid);
+        cl.map_shared_rank(part, r)[slot * kPkMaxCta + q].w[w] = v;
     }
     cl.sync();
-    // lane r < ncta of warp 0 takes rank r's part
+    // lane r of each eight of warp 0 takes rank r's part
     if (wid == 0) {
-        const bool in = lane < p.ncta;
-        const PkPart *pr = cl.map_shared_rank(part, in ? lane : 0) + slot;
-        double m = in ? pr->mx : -INFINITY, M = m, R[kPkStats];
-        for (int o = 16; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
-        const int top = __ffs((int)__ballot_sync(0xFFFFFFFFu, m == M)) - 1;
-        const double f = in && m > -INFINITY ? exp(m - M) : 0.0;
-        const int Er = in ? pr->E : 0;
-        const double Jr = in ? pr->J : 0.0;
+        const bool in = (lane & 7) < p.ncta;
+        const double *pw = part[slot * kPkMaxCta + (in ? lane & 7 : 0)].w;
+        const double ei = pw[kPkStats + 4];
+        const PkRef rr{pw[kPkStats], pw[kPkStats + 1], pw[kPkStats + 2], pw[kPkStats + 3],
+                       __double2loint(ei), __double2hiint(ei)};
+        double R[kPkStats];
 #pragma unroll
-        for (int j = 0; j < kPkStats; ++j) R[j] = f > 0.0 ? f * pr->R[j] : 0.0;
+        for (int j = 0; j < kPkStats; ++j) R[j] = pw[j];
+        const bool on = in && rr.E >= 0;
+        const double m = on ? fma(-dc, (double)(rr.mid - er), rr.ah) + rr.ln : -INFINITY;
+        double M = m;
+        for (int o = 4; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
+        const int top = __ffs((int)__ballot_sync(0xFFFFFFFFu, m == M)) - 1;
+        // relative to the leading CTA's reference
+        const double h0 = __shfl_sync(0xFFFFFFFFu, rr.ah, top), l0 = __shfl_sync(0xFFFFFFFFu, rr.al, top);
+        const int mid0 = __shfl_sync(0xFFFFFFFFu, rr.mid, top);
+        const int E0 = __shfl_sync(0xFFFFFFFFu, rr.E, top);
+        const double J0 = __shfl_sync(0xFFFFFFFFu, rr.J, top);
+        const double f = exp(fma(-dc, (double)(rr.mid - mid0), (rr.ah - h0) + (rr.al - l0)));
+#pragma unroll
+        for (int j = 0; j < kPkStats; ++j) R[j] = on ? f * R[j] : 0.0;
+        const int Er = on ? rr.E : E0;
+        const double Jr = on ? rr.J : J0;
         // the means about the leading CTA's references
-        const int E0 = __shfl_sync(0xFFFFFFFFu, Er, top);
-        const double J0 = __shfl_sync(0xFFFFFFFFu, Jr, top);
         double z[3] = {R[0], fma(R[0], (double)(Er - E0), R[1]), fma(R[0], Jr - J0, R[3])};
 #pragma unroll
         for (int j = 0; j < 3; ++j)
-            for (int o = 16; o > 0; o >>= 1) z[j] += __shfl_xor_sync(0xFFFFFFFFu, z[j], o);
+            for (int o = 4; o > 0; o >>= 1) z[j] += __shfl_xor_sync(0xFFFFFFFFu, z[j], o);
         const double iz = 1.0 / z[0];
         pk_shift(R, (double)(Er - E0) - z[1] * iz, (Jr - J0) - z[2] * iz);
         double cv = R[4], th = R[5];
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = 4; o > 0; o >>= 1) {
             cv += __shfl_xor_sync(0xFFFFFFFFu, cv, o);
             th += __shfl_xor_sync(0xFFFFFFFFu, th, o);
         }
@@ -417,28 +488,29 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
 
 // One cluster per data set: bisection on the sign of dC/dDelta in [lo, hi].
 // Every CTA of a cluster holds the same combined sums, so all take the same
-// steps; a final cluster barrier keeps each CTA's shared memory alive until
-// the others have read it.
+// steps.  A cluster barrier before the first step: a CTA's shared memory may be
+// written by the others only once it runs.
 __global__ void __launch_bounds__(kPkStepThreads)
 peak_kernel(PkBlocks bl, PkPlan p, int nE, double beta, double lo, double hi, int n_iter,
             double *res, int *bad)
 {
     __shared__ double sh[24];
     __shared__ int shi[4];
-    __shared__ PkPart part[2];
+    __shared__ PkPart part[2 * kPkMaxCta];  // [slot][rank]
     cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
     const int q = (int)cl.block_rank(), d = blockIdx.x / p.ncta;
     int slot = 0;
     // Exponents move by |c - s| |E - E_r| from the interval's middle to its
     // ends: where that is at most 200 (weights within e^+-200 of the reference),
     // the largest exponent is found once
     const bool wide = 0.5 * beta * (hi - lo) * nE > 200.0;
-    double mx = -INFINITY, z0;
-    int at = -1;
+    PkRef ref;
+    double z0;
     bool find = true;
     auto third_at = [&](double delta, double &cov) {
         double t;
-        pk_moments(cl, part, slot, bl, p, d, nE, beta * delta, find, mx, at, sh, shi, cov, t, z0);
+        pk_moments(cl, part, slot, bl, p, d, nE, beta * delta, find, ref, sh, shi, cov, t, z0);
         find = wide;
         return t;
     };
@@ -446,7 +518,6 @@ peak_kernel(PkBlocks bl, PkPlan p, int nE, double beta, double lo, double hi, in
     const double t_lo = third_at(lo, cov), t_hi = third_at(hi, cov);
     if (!(t_lo > 0.0 && t_hi < 0.0)) {
         if (q == 0 && threadIdx.x == 0) bad[d] = 1;
-        cl.sync();
         return;
     }
     for (int i = 0; i < n_iter; ++i) {
@@ -460,7 +531,6 @@ peak_kernel(PkBlocks bl, PkPlan p, int nE, double beta, double lo, double hi, in
         res[2 * d] = ds;
         res[2 * d + 1] = -beta * (cov / z0);
     }
-    cl.sync();
 }
 
 // ---------------------------------------------------- equal height, barrier
@@ -746,7 +816,7 @@ static cudaError_t cluster_config(const void *kernel, int n_sets, int threads, i
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int ncta = std::max(1, std::min(std::min(8, max_cta), nsm / std::max(n_sets, 1)));
+    int ncta = std::max(1, std::min(std::min(kPkMaxCta, max_cta), nsm / std::max(n_sets, 1)));
     for (; ncta > 1; --ncta) {
         attr[0].val.clusterDim.x = (unsigned)ncta;
         cfg.gridDim = dim3((unsigned)(n_sets * ncta));

@@ -222,3 +222,26 @@ def test_peak_blocks_of_bins_every_size(scale, jack):
     assert abs(got[2] - ref[0, 1]) <= 1e-10 * abs(ref[0, 1])
     np.testing.assert_allclose(got[4][:, 0], ref[1:, 0], rtol=0, atol=1e-9)
     np.testing.assert_allclose(got[4][:, 1], ref[1:, 1], rtol=1e-10)
+
+
+@pytest.mark.parametrize("hw", [0.5, 0.05])
+def test_peak_of_a_series_that_fills_few_bins_of_a_wide_window(hw):
+    """61 of 262145 bins hold samples, weights only there: exponents relative to
+    the window's middle bin are some 5e5, those that matter differ by a few.
+    Single bins (wide interval) and blocks of 32.  C* against binary128 at the
+    returned Delta*: E_J is one integer per bin, so nothing but the sums' own
+    rounding counts, some tens of units of 1.1e-16."""
+    rng = np.random.default_rng(2)
+    V, lo = 64 ** 3, 250000
+    e = np.arange(lo, lo + 61)
+    x = (e - lo) / 60.0
+    lnW = np.zeros(V + 1)
+    lnW[lo:lo + 61] = -2.0 * e + 3.0 * ((x - 0.25) * (x - 0.8)) ** 2 / 0.01
+    ed = np.repeat(e, rng.integers(200, 1000, 61))
+    ed = ed[: ed.size // 50 * 50].reshape(50, -1)
+    ej = -3 * (ed - lo)
+    ds, _, cs, _, _ = muca().find_peak(dev(ej), dev(ed), lnW, 0, 1.0, 2.0 - hw, 2.0 + hw)
+    want = oracle.reweight_q(ej, ed, 0 * ed, lnW, 0, 1.0, V, [ds])[0, 2]
+    assert abs(cs - want) <= 3e-14 * abs(want), abs(cs / want - 1)
+    near = oracle.reweight_q(ej, ed, 0 * ed, lnW, 0, 1.0, V, [ds - 1e-4 * hw, ds + 1e-4 * hw])[:, 2]
+    assert (near < want).all()
