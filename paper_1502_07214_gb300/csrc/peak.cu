@@ -111,11 +111,11 @@ constexpr int kPkThreads = 256;
 constexpr int kPkStats = 6;    // n, n r, n r^2, n J, n J r, n J r^2 (J about the block's mean)
 constexpr int kPkDegMax = 20;
 constexpr int kPkMaxB = 512;
-constexpr int kPkStepThreads = 64;
+constexpr int kPkFew = 64, kPkMany = 256;  // threads per CTA of a step
 constexpr int kPkMaxCta = 8;   // CTAs per cluster
 
 struct PkPlan {
-    int B, nblk, deg, ncta, per, slots;  // slots = ncta kPkStepThreads per
+    int B, nblk, deg, ncta, threads, per, slots;  // slots = ncta threads per
     double slope;
 };
 
@@ -141,11 +141,11 @@ PkPlan pk_plan(double c_lo, double c_hi, int nE)
     return p;
 }
 
-// Thread g of a set's ncta kPkStepThreads takes blocks g per .. g per + per - 1,
-// the i-th at slot i ncta kPkStepThreads + g.
+// Thread g of a set's ncta threads takes blocks g per .. g per + per - 1, the
+// i-th at slot i ncta threads + g.
 __host__ __device__ inline int pk_slot(const PkPlan &p, int b)
 {
-    return (b % p.per) * (p.ncta * kPkStepThreads) + b / p.per;
+    return (b % p.per) * (p.ncta * p.threads) + b / p.per;
 }
 
 // Per set and slot: coefficients [deg + 1][kPkStats], a_b = ah + al, the
@@ -156,10 +156,12 @@ struct PkBlocks {
     int *E;
 };
 
+// Coefficients per block: of a single bin n alone, its other sums are zero.
+int pk_coefs(const PkPlan &p) { return p.B == 1 ? 1 : kPkStats * (p.deg + 1); }
+
 size_t pk_block_bytes(const PkPlan &p, int n_sets)
 {
-    return (size_t)n_sets * p.slots *
-           ((kPkStats * (p.deg + 1) + 4) * sizeof(double) + sizeof(int));
+    return (size_t)n_sets * p.slots * ((pk_coefs(p) + 4) * sizeof(double) + sizeof(int));
 }
 
 PkBlocks pk_block_layout(const PkPlan &p, int n_sets, char *mem)
@@ -167,7 +169,7 @@ PkBlocks pk_block_layout(const PkPlan &p, int n_sets, char *mem)
     const size_t n = (size_t)n_sets * p.slots;
     PkBlocks b;
     b.coef = (double *)mem;
-    b.ah = b.coef + n * kPkStats * (p.deg + 1);
+    b.ah = b.coef + n * pk_coefs(p);
     b.al = b.ah + n;
     b.mj = b.al + n;
     b.ln = b.mj + n;
@@ -183,6 +185,35 @@ __constant__ double pk_inv[kPkDegMax + 1] = {
 __device__ __forceinline__ int pk_mid(const PkPlan &p, int b, int nE)
 {
     return min(b * p.B + p.B / 2, nE - 1);
+}
+
+// a_b of the bin `ref` relative to the bin `er`, as a pair: the product and the
+// differences without rounding.
+__device__ __forceinline__ void pk_exponent(double slope, int ref, int er, const double *lnW,
+                                            double &ah, double &al)
+{
+    const double lref = lnW[ref], l0 = lnW[er];
+    const double x = (double)(ref - er), a1 = -__dmul_rn(slope, x), pe = fma(slope, x, a1);
+    const double l = __dsub_rn(lref, l0), bb = __dsub_rn(l, lref);
+    const double le = __dsub_rn(__dsub_rn(lref, __dsub_rn(l, bb)), __dadd_rn(l0, bb));
+    const double h = __dsub_rn(a1, l), u = __dsub_rn(h, a1);
+    const double he = __dsub_rn(__dsub_rn(a1, __dsub_rn(h, u)), __dadd_rn(l, u));
+    ah = h;
+    al = he - (pe + le);
+}
+
+// Blocks of one bin, a thread each: n is their only statistic.
+__global__ void pk_single_kernel(const double *__restrict__ n_all, const double *__restrict__ mj_all,
+                                 const double *__restrict__ lnW, int nE, PkPlan p, PkBlocks out)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x, d = blockIdx.y;
+    if (e >= nE) return;
+    const double n = n_all[(size_t)d * nE + e];
+    const size_t slot = (size_t)d * p.slots + pk_slot(p, e);
+    out.ln[slot] = n > 0.0 ? log(n) : -INFINITY;
+    out.coef[slot] = n;
+    out.mj[slot] = mj_all[(size_t)d * nE + e];
+    pk_exponent(p.slope, e, nE / 2, lnW, out.ah[slot], out.al[slot]);
 }
 
 // One (block, data set) per CTA of 128 threads.
@@ -256,15 +287,7 @@ pk_coef_kernel(const double *__restrict__ n_all, const double *__restrict__ mj_a
     sj = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
     const double jb = jref + sj / sn;
     if (i == 0) {
-        // a_b: the product and the differences without rounding, as a pair
-        const int er = nE / 2;
-        const double x = (double)(ref - er), a1 = -__dmul_rn(p.slope, x), pe = fma(p.slope, x, a1);
-        const double l0 = lnW[er], l = __dsub_rn(lref, l0), bb = __dsub_rn(l, lref);
-        const double le = __dsub_rn(__dsub_rn(lref, __dsub_rn(l, bb)), __dadd_rn(l0, bb));
-        const double h = __dsub_rn(a1, l), u = __dsub_rn(h, a1);
-        const double he = __dsub_rn(__dsub_rn(a1, __dsub_rn(h, u)), __dadd_rn(l, u));
-        out.ah[slot] = h;
-        out.al[slot] = he - (pe + le);
+        pk_exponent(p.slope, ref, nE / 2, lnW, out.ah[slot], out.al[slot]);
         out.mj[slot] = jb;
         out.ln[slot] = log(n[ref]);
         out.E[slot] = ref;
@@ -314,8 +337,10 @@ struct PkRef {
 };
 
 // One CTA's part of a step: its sums R relative to the exponent of its reference
-// block, about (E, J) of that block, then the block's ah, al, ln, J, (E, mid).
+// block, about (E, J) of that block, then (in a step that finds it) the block's
+// ah, al, ln, J, (E, mid).
 constexpr int kPkWords = kPkStats + 5;
+constexpr int kPkSums = kPkMany / 32 * kPkStats;
 struct PkPart {
     double w[kPkWords];
 };
@@ -339,15 +364,17 @@ __device__ __forceinline__ void pk_shift(double (&R)[kPkStats], double dE, doubl
 // (slots alternate, so one cluster barrier per step suffices); every thread gets
 // the result.
 // ref: the heaviest of the CTA's blocks, found anew when `find` is set, else kept
-// as a fixed reference.
+// as a fixed reference; peer: that of rank lane % 8, in warp 0.
+// SINGLE: blocks of one bin, whose only statistic is n.
 // Results: the moments times z = sum n (the sign of the third is all that a
 // step needs).
+template <int NT, bool SINGLE>
 __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const PkBlocks &bl,
                            const PkPlan &p, int d, int nE, double c, bool find, PkRef &ref,
-                           double *sh, int *shi, double &cov, double &third, double &z0)
+                           PkRef &peer, double *sh, int *shi, double &cov, double &third, double &z0)
 {
     const int q = (int)cl.block_rank(), t = (int)threadIdx.x, lane = t & 31, wid = t >> 5;
-    const int g = q * kPkStepThreads + t, gs = p.ncta * kPkStepThreads;
+    const int g = q * NT + t, gs = p.ncta * NT;
     const size_t base = (size_t)d * p.slots, stride = (size_t)(gridDim.x / p.ncta) * p.slots;
     const double dc = c - p.slope, x = -dc * (0.5 * p.B);
     const int er = nE / 2;
@@ -378,7 +405,7 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
             shi[wid] = at;
         }
         __syncthreads();
-        for (int i = 0; i < kPkStepThreads / 32; ++i)
+        for (int i = 0; i < NT / 32; ++i)
             if (sh[i] > mx || (sh[i] == mx && shi[i] > at)) {
                 mx = sh[i];
                 at = shi[i];
@@ -386,7 +413,8 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
         ref = PkRef{0.0, 0.0, -INFINITY, 0.0, er, -1};
         if (at >= 0) {
             const size_t k = base + pk_slot(p, at);
-            ref = PkRef{bl.ah[k], bl.al[k], bl.ln[k], bl.mj[k], pk_mid(p, at, nE), bl.E[k]};
+            ref = PkRef{bl.ah[k], bl.al[k], bl.ln[k], bl.mj[k], pk_mid(p, at, nE),
+                        SINGLE ? at : bl.E[k]};
         }
     }
     double S[kPkStats];
@@ -397,20 +425,35 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
         const size_t k = base + (size_t)i * gs + g;
         // loaded together (slots past the last block are allocated, and not used)
         const double ln = bl.ln[k], ah = bl.ah[k], al = bl.al[k], mj = bl.mj[k];
-        const int E = bl.E[k];
+        const double n = SINGLE ? bl.coef[k] : 0.0;
+        const int E = SINGLE ? b : bl.E[k];
         if (b >= p.nblk || ln == -INFINITY) continue;
         const double A = exp(fma(-dc, (double)(pk_mid(p, b, nE) - ref.mid), (ah - ref.ah) + (al - ref.al)));
         if (!(A > 0.0)) continue;
-        double R[kPkStats];
-#pragma unroll
-        for (int j = 0; j < kPkStats; ++j) R[j] = bl.coef[(size_t)(p.deg * kPkStats + j) * stride + k];
-        for (int u = p.deg - 1; u >= 0; --u)
+        if constexpr (SINGLE) {
+            const double dE = (double)(E - ref.E), dJ = mj - ref.J, w = A * n;
+            const double we = w * dE, wee = we * dE;
+            S[0] += w;
+            S[1] += we;
+            S[2] += wee;
+            S[3] = fma(w, dJ, S[3]);
+            S[4] = fma(we, dJ, S[4]);
+            S[5] = fma(wee, dJ, S[5]);
+        } else {
+            double R[kPkStats];
 #pragma unroll
             for (int j = 0; j < kPkStats; ++j)
-                R[j] = fma(R[j], x, bl.coef[(size_t)(u * kPkStats + j) * stride + k]);
-        pk_shift(R, (double)(E - ref.E), mj - ref.J);
+                R[j] = bl.coef[(size_t)(p.deg * kPkStats + j) * stride + k];
+            // (unrolled: the coefficients of several orders are on their way at once)
+#pragma unroll 4
+            for (int u = p.deg - 1; u >= 0; --u)
 #pragma unroll
-        for (int j = 0; j < kPkStats; ++j) S[j] = fma(A, R[j], S[j]);
+                for (int j = 0; j < kPkStats; ++j)
+                    R[j] = fma(R[j], x, bl.coef[(size_t)(u * kPkStats + j) * stride + k]);
+            pk_shift(R, (double)(E - ref.E), mj - ref.J);
+#pragma unroll
+            for (int j = 0; j < kPkStats; ++j) S[j] = fma(A, R[j], S[j]);
+        }
     }
 #pragma unroll
     for (int j = 0; j < kPkStats; ++j)
@@ -422,11 +465,13 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
     __syncthreads();
     // this CTA's part to every CTA of the cluster, a word per thread (reading the
     // others' parts instead waits for distributed shared memory once more)
-    for (int i = t; i < kPkWords * p.ncta; i += kPkStepThreads) {
-        const int r = i / kPkWords, w = i - r * kPkWords;
+    const int words = find ? kPkWords : kPkStats;
+    for (int i = t; i < 8 * words; i += NT) {
+        const int r = i & 7, w = i >> 3;
+        if (r >= p.ncta) continue;
         double v = 0.0;
         if (w < kPkStats)
-            for (int k = 0; k < kPkStepThreads / 32; ++k) v += sh[k * kPkStats + w];
+            for (int k = 0; k < NT / 32; ++k) v += sh[k * kPkStats + w];
         else
             v = w == kPkStats       ? ref.ah
                 : w == kPkStats + 1 ? ref.al
@@ -440,9 +485,12 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
     if (wid == 0) {
         const bool in = (lane & 7) < p.ncta;
         const double *pw = part[slot * kPkMaxCta + (in ? lane & 7 : 0)].w;
-        const double ei = pw[kPkStats + 4];
-        const PkRef rr{pw[kPkStats], pw[kPkStats + 1], pw[kPkStats + 2], pw[kPkStats + 3],
-                       __double2loint(ei), __double2hiint(ei)};
+        if (find) {
+            const double ei = pw[kPkStats + 4];
+            peer = PkRef{pw[kPkStats], pw[kPkStats + 1], pw[kPkStats + 2], pw[kPkStats + 3],
+                         __double2loint(ei), __double2hiint(ei)};
+        }
+        const PkRef &rr = peer;
         double R[kPkStats];
 #pragma unroll
         for (int j = 0; j < kPkStats; ++j) R[j] = pw[j];
@@ -474,44 +522,46 @@ __device__ void pk_moments(cg::cluster_group &cl, PkPart *part, int &slot, const
             th += __shfl_xor_sync(0xFFFFFFFFu, th, o);
         }
         if (lane == 0) {
-            sh[16] = cv;
-            sh[17] = th;
-            sh[18] = z[0];
+            sh[kPkSums] = cv;
+            sh[kPkSums + 1] = th;
+            sh[kPkSums + 2] = z[0];
         }
     }
     slot ^= 1;
     __syncthreads();
-    cov = sh[16];
-    third = sh[17];
-    z0 = sh[18];
+    cov = sh[kPkSums];
+    third = sh[kPkSums + 1];
+    z0 = sh[kPkSums + 2];
 }
 
 // One cluster per data set: bisection on the sign of dC/dDelta in [lo, hi].
 // Every CTA of a cluster holds the same combined sums, so all take the same
 // steps.  A cluster barrier before the first step: a CTA's shared memory may be
 // written by the others only once it runs.
-__global__ void __launch_bounds__(kPkStepThreads)
+template <int NT, bool SINGLE>
+__global__ void __launch_bounds__(NT)
 peak_kernel(PkBlocks bl, PkPlan p, int nE, double beta, double lo, double hi, int n_iter,
             double *res, int *bad)
 {
-    __shared__ double sh[24];
-    __shared__ int shi[4];
+    __shared__ double sh[kPkSums + 3];  // the warps' sums, then the results
+    __shared__ int shi[kPkMany / 32];
     __shared__ PkPart part[2 * kPkMaxCta];  // [slot][rank]
     cg::cluster_group cl = cg::this_cluster();
     cl.sync();
     const int q = (int)cl.block_rank(), d = blockIdx.x / p.ncta;
     int slot = 0;
-    // Exponents move by |c - s| |E - E_r| from the interval's middle to its
-    // ends: where that is at most 200 (weights within e^+-200 of the reference),
-    // the largest exponent is found once
-    const bool wide = 0.5 * beta * (hi - lo) * nE > 200.0;
-    PkRef ref;
+    // Exponents move by at most beta (hi - lo) |E - E'| in what is left of the
+    // interval: once that is 400 (the weights within e^+-400 of the reference) or
+    // less, the heaviest block is not looked for again
+    PkRef ref, peer;
     double z0;
-    bool find = true;
+    bool first = true;
     auto third_at = [&](double delta, double &cov) {
         double t;
-        pk_moments(cl, part, slot, bl, p, d, nE, beta * delta, find, ref, sh, shi, cov, t, z0);
-        find = wide;
+        const bool find = first || beta * (hi - lo) * nE > 400.0;
+        first = false;
+        pk_moments<NT, SINGLE>(cl, part, slot, bl, p, d, nE, beta * delta, find, ref, peer, sh, shi,
+                               cov, t, z0);
         return t;
     };
     double cov;
@@ -860,17 +910,29 @@ extern "C" int muca_find_peak(const int32_t *e_j, const int32_t *e_d, int64_t n_
     const size_t b_res = al((size_t)2 * n_sets * sizeof(double));
     const size_t b_bad = al((size_t)(n_sets + 1) * sizeof(int));
     // blocks of bins, spread over the CTAs of each set's cluster: at least 16
-    // blocks per CTA (below that a step is its barriers)
+    // blocks per CTA (below that a step is its barriers), and 256 threads per CTA
+    // instead of 64 where those would take more than two blocks each (latency:
+    // 101 sets of 4097 bins in blocks of 32 2.5 -> 1.5 ms, of 1729 single bins
+    // on 8 CTAs 0.81 -> 0.71 ms; 513 single bins on 8 CTAs 0.60 on 64 threads,
+    // 0.68 on 256)
     PkPlan plan = pk_plan(beta * delta_lo, beta * delta_hi, n_e);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    cudaError_t ce = cluster_config((const void *)peak_kernel, n_sets, kPkStepThreads,
+    const bool single = plan.B == 1;
+    auto kernel = single ? &peak_kernel<kPkFew, true> : &peak_kernel<kPkFew, false>;
+    plan.threads = kPkFew;
+    cudaError_t ce = cluster_config((const void *)kernel, n_sets, plan.threads,
                                     (plan.nblk + 15) / 16, st, cfg, attr);
+    if (ce == cudaSuccess && plan.nblk > 2 * kPkFew * (int)attr[0].val.clusterDim.x) {
+        kernel = single ? &peak_kernel<kPkMany, true> : &peak_kernel<kPkMany, false>;
+        plan.threads = kPkMany;
+        ce = cluster_config((const void *)kernel, n_sets, plan.threads, kPkMaxCta, st, cfg, attr);
+    }
     if (ce != cudaSuccess)
         return pk_fail(MUCA_ERR_CUDA, std::string("cluster configuration: ") + cudaGetErrorString(ce));
     plan.ncta = (int)attr[0].val.clusterDim.x;
-    plan.per = (plan.nblk + plan.ncta * kPkStepThreads - 1) / (plan.ncta * kPkStepThreads);
-    plan.slots = plan.ncta * kPkStepThreads * plan.per;
+    plan.per = (plan.nblk + plan.ncta * plan.threads - 1) / (plan.ncta * plan.threads);
+    plan.slots = plan.ncta * plan.threads * plan.per;
     const size_t b_w = al(pk_block_bytes(plan, n_sets));
     char *p = nullptr;
     cudaMemPool_t pool = nullptr;
@@ -913,10 +975,13 @@ extern "C" int muca_find_peak(const int32_t *e_j, const int32_t *e_d, int64_t n_
         dim3 g2((unsigned)((n_e + 255) / 256), (unsigned)n_sets);
         jk_stats_kernel<<<g2, 256, 0, st>>>(cnt, sej, n_blocks, n_e, n_all, mj_all);
         PCK(cudaGetLastError());
-        pk_coef_kernel<<<dim3((unsigned)plan.nblk, (unsigned)n_sets), 128, 0, st>>>(
-            n_all, mj_all, d_lnW, n_e, plan, blocks);
+        if (single)
+            pk_single_kernel<<<g2, 256, 0, st>>>(n_all, mj_all, d_lnW, n_e, plan, blocks);
+        else
+            pk_coef_kernel<<<dim3((unsigned)plan.nblk, (unsigned)n_sets), 128, 0, st>>>(
+                n_all, mj_all, d_lnW, n_e, plan, blocks);
         PCK(cudaGetLastError());
-        PCK(cudaLaunchKernelEx(&cfg, peak_kernel, blocks, plan, (int)n_e, beta, delta_lo, delta_hi,
+        PCK(cudaLaunchKernelEx(&cfg, kernel, blocks, plan, (int)n_e, beta, delta_lo, delta_hi,
                                (int)n_iter, d_res, d_bad + 1));
     }
     PCK(cudaMemcpyAsync(res.data(), d_res, res.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
