@@ -140,15 +140,19 @@ cudaError_t launch_sweeps_scan(int L, const GroupDev *groups_dev, const BlockDes
 // Site-per-lane launch (rows.cu), 3 <= L <= 64, with or without couplings per
 // bond: a walker's row is cut into seg segments of `lanes` consecutive sites,
 // one site per lane, and a block (one warp) serves per_warp = 32 / lanes
-// of its W walkers.  One launch per group; seg = 0: not supported.
+// of its W walkers; seg = 0: not supported.
 struct RowShape {
     int seg, lanes, per_warp;
 };
 RowShape rows_shape(int L, int W);
 // Words per row of a lattice kept walker by walker.
 int rows_lattice_words(int L);
-cudaError_t launch_sweeps_rows(const GroupDev &g, uint32_t seed, uint64_t sweep0, int n_sweeps,
-                               int64_t ts_pos, bool record, cudaStream_t st);
+// One launch sweeps up to kRowsMaxGroups groups of one kind (segments, row width
+// in shared memory, couplings or not).
+constexpr int kRowsMaxGroups = 128;
+int rows_kind(const GroupDev &g);
+cudaError_t launch_sweeps_rows(const GroupDev *const *g, int n, uint32_t seed, uint64_t sweep0,
+                               int n_sweeps, int64_t ts_pos, bool record, cudaStream_t st);
 // Sweeps of groups with couplings per bond that the site-per-lane kernel does
 // not cover (bonds.cu, L = 2): blocks of one warp, one thread per walker,
 // BlockDesc.nw <= 32 walkers (P = 1).

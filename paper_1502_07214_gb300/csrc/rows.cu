@@ -51,6 +51,7 @@
 //   couplings, L = 24, 4096 walkers, 50 and merge     120 -> 23.4 ms
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "muca_internal.h"
@@ -575,6 +576,37 @@ sweep_rows_kernel(const __grid_constant__ GroupDev g, int lanes, uint32_t seed, 
                                    sweep0, n_sweeps, ts_pos, record);
 }
 
+// The groups of one launch, in kernel parameters (32764 bytes at most; from there
+// every block reads its group's values uniformly): group i's blocks are
+// first[i] .. first[i + 1] - 1.  One launch for up to 128 groups of a kind: a
+// launch per group keeps at most 32 of them on the GPU at a time (one per stream).
+//   us per sweep of 128 groups of 32 walkers, L = 8: 66 -> 16, of 256: 132 -> 22;
+//   100 groups of 8 walkers, L = 32: 905 -> 274; 24 groups of 512, L = 8 .. 32, 60
+//   sweeps and merge 43.5 -> 42.1 ms
+struct RowsList {
+    GroupDev g[kRowsMaxGroups];
+    int first[kRowsMaxGroups + 1], lanes[kRowsMaxGroups];
+    int n;
+};
+static_assert(sizeof(RowsList) <= 32000, "kernel parameters");
+
+template <int SEG, int PITCH, bool BONDS>
+__global__ void __launch_bounds__(32, 16)
+sweep_rows_list_kernel(const __grid_constant__ RowsList list, uint32_t seed, uint64_t sweep0,
+                       int n_sweeps, int64_t ts_pos, int record)
+{
+    extern __shared__ __align__(16) uint32_t s_rows[];
+    // the last group with first <= block
+    int i = 0;
+#pragma unroll
+    for (int step = kRowsMaxGroups / 2; step > 0; step /= 2)
+        i += i + step < list.n && list.first[i + step] <= (int)blockIdx.x ? step : 0;
+    const int per_warp = 32 / list.lanes[i];
+    rows_sweeps<SEG, PITCH, BONDS>(list.g[i], list.lanes[i], per_warp,
+                                   ((int)blockIdx.x - list.first[i]) * per_warp, s_rows, seed,
+                                   sweep0, n_sweeps, ts_pos, record);
+}
+
 }  // namespace
 
 // Segments and lanes of a row of L sites, for a group of W walkers.  Rows of up
@@ -606,31 +638,55 @@ static size_t rows_bytes_for(int L, const RowShape &s)
 }
 
 namespace {
-template <int SEG, int PITCH>
-void launch(const GroupDev &g, const RowShape &sh, int blocks, size_t smem, uint32_t seed,
+template <int SEG, int PITCH, bool BONDS>
+void launch(const GroupDev *const *g, const RowShape *sh, int n, size_t smem, uint32_t seed,
             uint64_t sweep0, int n_sweeps, int64_t ts_pos, int rec, cudaStream_t st)
 {
-    if (g.jmax > 0)
-        sweep_rows_kernel<SEG, PITCH, true><<<blocks, 32, smem, st>>>(g, sh.lanes, seed, sweep0,
-                                                                      n_sweeps, ts_pos, rec);
-    else
-        sweep_rows_kernel<SEG, PITCH, false><<<blocks, 32, smem, st>>>(g, sh.lanes, seed, sweep0,
-                                                                       n_sweeps, ts_pos, rec);
+    auto blocks = [&](int i) { return (g[i]->W + sh[i].per_warp - 1) / sh[i].per_warp; };
+    if (n == 1) {
+        sweep_rows_kernel<SEG, PITCH, BONDS><<<blocks(0), 32, smem, st>>>(
+            *g[0], sh[0].lanes, seed, sweep0, n_sweeps, ts_pos, rec);
+        return;
+    }
+    RowsList list;
+    list.n = n;
+    list.first[0] = 0;
+    for (int i = 0; i < n; ++i) {
+        list.g[i] = *g[i];
+        list.lanes[i] = sh[i].lanes;
+        list.first[i + 1] = list.first[i] + blocks(i);
+    }
+    sweep_rows_list_kernel<SEG, PITCH, BONDS><<<list.first[n], 32, smem, st>>>(
+        list, seed, sweep0, n_sweeps, ts_pos, rec);
 }
 }  // namespace
 
-cudaError_t launch_sweeps_rows(const GroupDev &g, uint32_t seed, uint64_t sweep0, int n_sweeps,
-                               int64_t ts_pos, bool record, cudaStream_t st)
+int rows_kind(const GroupDev &g)
+{
+    return (rows_shape(g.L, g.W).seg * 100 + rows_pitch(g.L)) * 2 + (g.jmax > 0);
+}
+
+cudaError_t launch_sweeps_rows(const GroupDev *const *g, int n, uint32_t seed, uint64_t sweep0,
+                               int n_sweeps, int64_t ts_pos, bool record, cudaStream_t st)
 {
     if (n_sweeps <= 0) return cudaSuccess;
-    const RowShape sh = rows_shape(g.L, g.W);
-    if (sh.seg == 0) return cudaErrorInvalidValue;
-    const int blocks = (g.W + sh.per_warp - 1) / sh.per_warp, rec = record ? 1 : 0;
-    const size_t smem = rows_bytes_for(g.L, sh);  // at most 16 KB: no opt-in
-    switch (sh.seg * 100 + rows_pitch(g.L)) {
-#define MUCA_ROWS_LAUNCH(S, P)                                                          \
-    case S * 100 + P:                                                                   \
-        launch<S, P>(g, sh, blocks, smem, seed, sweep0, n_sweeps, ts_pos, rec, st);     \
+    if (n < 1 || n > kRowsMaxGroups) return cudaErrorInvalidValue;
+    RowShape sh[kRowsMaxGroups];
+    size_t smem = 0;  // at most 16 KB: no opt-in
+    const int kind = rows_kind(*g[0]);
+    for (int i = 0; i < n; ++i) {
+        sh[i] = rows_shape(g[i]->L, g[i]->W);
+        if (sh[i].seg == 0 || rows_kind(*g[i]) != kind) return cudaErrorInvalidValue;
+        smem = std::max(smem, rows_bytes_for(g[i]->L, sh[i]));
+    }
+    const int rec = record ? 1 : 0;
+    switch (kind) {
+#define MUCA_ROWS_LAUNCH(S, P)                                                                \
+    case (S * 100 + P) * 2:                                                                   \
+        launch<S, P, false>(g, sh, n, smem, seed, sweep0, n_sweeps, ts_pos, rec, st);         \
+        break;                                                                                \
+    case (S * 100 + P) * 2 + 1:                                                               \
+        launch<S, P, true>(g, sh, n, smem, seed, sweep0, n_sweeps, ts_pos, rec, st);          \
         break;
         MUCA_ROWS_LAUNCH(1, 16)
         MUCA_ROWS_LAUNCH(1, 32)

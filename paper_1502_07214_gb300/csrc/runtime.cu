@@ -102,10 +102,11 @@ struct muca_ctx {
         size_t smem;
     };
     std::vector<ScanRange> scan_ranges;
-    // the groups of the site-per-lane kind, one launch each, largest L first
-    std::vector<int> rows_groups;
-    // streams of the row-scan ranges' and the site-per-lane groups' launches, in
-    // this order, taken in turn when there are more launches than streams
+    // the launches of the site-per-lane kind: groups of one rows_kind each, the
+    // launches and the groups in them by falling L
+    std::vector<std::vector<int>> rows_launches;
+    // streams of the row-scan ranges' and the site-per-lane launches, in this
+    // order, taken in turn when there are more launches than streams
     std::vector<cudaStream_t> range_streams;
     std::vector<cudaEvent_t> range_events;
 };
@@ -452,14 +453,14 @@ int bonds_walkers_per_warp(int W)
 
 int build_blocks(muca_ctx *ctx)
 {
-    ctx->rows_groups.clear();
+    std::vector<int> rows;
     std::vector<BlockDesc> b[kKinds];
     size_t sm[kKinds] = {};
     for (size_t gi = 0; gi < ctx->g.size(); ++gi) {
         const Group &g = ctx->g[gi];
         const int k = kind_of(g);
         if (k < 0) {
-            ctx->rows_groups.push_back((int)gi);
+            rows.push_back((int)gi);
             continue;
         }
         const size_t need = k == 0   ? stage_bytes_for(g.wpb)
@@ -473,8 +474,19 @@ int build_blocks(muca_ctx *ctx)
             b[k].push_back(BlockDesc{(int)gi, w0, std::min(wpb, g.W - w0), wpb, P});
     }
     // the site-per-lane launches: the longest (most rows per walker) first
-    std::stable_sort(ctx->rows_groups.begin(), ctx->rows_groups.end(),
+    std::stable_sort(rows.begin(), rows.end(),
                      [&](int x, int y) { return ctx->g[x].L > ctx->g[y].L; });
+    ctx->rows_launches.clear();
+    std::map<int, size_t> open;  // kind -> its launch that has room
+    for (int gi : rows) {
+        const int kind = rows_kind(dev_of(ctx->g[gi]));
+        auto it = open.find(kind);
+        if (it == open.end() || ctx->rows_launches[it->second].size() == (size_t)kRowsMaxGroups) {
+            open[kind] = ctx->rows_launches.size();
+            ctx->rows_launches.emplace_back();
+        }
+        ctx->rows_launches[open[kind]].push_back(gi);
+    }
     // Longest blocks first: when a launch needs more than one wave of blocks,
     // the blocks of the largest lattices (work per sweep: walkers x sites)
     // start first instead of forming the tail.  Row-scan blocks are grouped
@@ -499,7 +511,7 @@ int build_blocks(muca_ctx *ctx)
         CK(prepare_scan_kernel(rg.L, rg.smem));
     }
     while (ctx->range_streams.size() <
-           std::min(ctx->scan_ranges.size() + ctx->rows_groups.size(), kRangeStreams)) {
+           std::min(ctx->scan_ranges.size() + ctx->rows_launches.size(), kRangeStreams)) {
         cudaStream_t s = nullptr;
         cudaEvent_t e = nullptr;
         CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
@@ -533,7 +545,7 @@ int build_blocks(muca_ctx *ctx)
 // in use, otherwise forked over per-launch streams and joined.
 int launch_all(muca_ctx *ctx, int n_sweeps, bool record, cudaStream_t st)
 {
-    const size_t n_scan = ctx->scan_ranges.size(), n_range = n_scan + ctx->rows_groups.size();
+    const size_t n_scan = ctx->scan_ranges.size(), n_range = n_scan + ctx->rows_launches.size();
     int used = (int)n_range;
     for (int k = 0; k < 4; ++k) used += ctx->n_blocks[k] > 0;
     used += ctx->n_blocks[5] > 0;
@@ -549,8 +561,15 @@ int launch_all(muca_ctx *ctx, int n_sweeps, bool record, cudaStream_t st)
                                   rg.smem, ctx->seed, ctx->sweep, n_sweeps, ctx->ts_len, record,
                                   s));
         } else {
-            CK(launch_sweeps_rows(dev_of(ctx->g[ctx->rows_groups[i - n_scan]]), ctx->seed,
-                                  ctx->sweep, n_sweeps, ctx->ts_len, record, s));
+            GroupDev gd[kRowsMaxGroups];
+            const GroupDev *gp[kRowsMaxGroups];
+            int n = 0;
+            for (int gi : ctx->rows_launches[i - n_scan]) {
+                gd[n] = dev_of(ctx->g[gi]);
+                gp[n] = gd + n;
+                ++n;
+            }
+            CK(launch_sweeps_rows(gp, n, ctx->seed, ctx->sweep, n_sweeps, ctx->ts_len, record, s));
         }
     }
     for (size_t i = 0; fork && i < std::min(n_range, n_streams); ++i) {

@@ -118,3 +118,69 @@ def test_checkpoints_cross_lattice_layouts(L, tmp_path):
         got = c.get_state(0)
         assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
         c.close()
+
+
+def _groups_against_the_general_path(groups, bonds, n):
+    """All groups of one context on the site-per-lane kernel, and on the
+    lanes-per-walker kernel: state, histogram and series bit for bit."""
+    out = []
+    for kw in ({}, {"residency": muca().RES_GLOBAL, "walkers_per_block": 32}):
+        c = muca().Context(groups, seed=9, **kw)
+        for g, s in enumerate(groups):
+            V = s["L"] ** 3
+            if g in bonds:
+                c.set_bonds(g, bonds[g])
+            elif not kw:
+                assert c.get_config(g)[0] == muca().RES_ROWS
+            c.set_lnW(g, -1.5 * np.arange(V + 1) + wl.random_lnW(V + 1, g, scale=0.3))
+        c.reserve_timeseries(n)
+        c.sweep_iter(n, record=True)
+        out.append([(c.get_state(g), c.get_hist(g), c.get_timeseries(g))
+                    for g in range(len(groups))])
+        c.check_tallies()
+        c.close()
+    for g, (a, b) in enumerate(zip(*out)):
+        assert np.array_equal(a[0][0], b[0][0]) and np.array_equal(a[0][1], b[0][1]), g
+        assert np.array_equal(a[1], b[1]) and np.array_equal(a[2], b[2]), g
+
+
+@pytest.mark.parametrize("n_groups", [2, 5, 127, 128, 129, 300])
+def test_many_groups_share_launches(n_groups):
+    """One launch takes 128 groups: row lengths, walkers per warp and block
+    counts that differ from group to group."""
+    rng = np.random.default_rng(n_groups)
+    groups = [{"L": int(L), "T": float(T), "n_walkers": int(W)} for L, T, W in
+              zip(rng.integers(3, 10, n_groups), rng.choice([0.9, 1.4182, 3.0], n_groups),
+                  rng.integers(1, 40, n_groups))]
+    _groups_against_the_general_path(groups, {}, 3)
+
+
+def test_groups_of_every_kind_in_one_context():
+    """Row widths, segment counts, couplings and L = 2 (no site-per-lane rows)."""
+    Ls = [3, 16, 17, 32, 33, 48, 49, 64, 16, 20, 33, 3, 12, 48, 50]
+    groups = [{"L": L, "T": 1.4182, "n_walkers": 3 + i} for i, L in enumerate(Ls)]
+    groups.append({"L": 36, "T": 1.4182, "n_walkers": 620})
+    bonds = {i: wl.random_bonds(groups[i]["L"], 5, 3, seed=i) for i in (1, 8, 9, 10, 14)}
+    _groups_against_the_general_path(groups, bonds, 2)
+
+
+def test_many_small_groups_run_side_by_side():
+    """256 groups of 32 walkers fill a sixth of the chip: a sweep of them takes
+    little longer than one of 24 such groups (measured 1.5 times; 7.8 times when
+    groups beyond the 32nd waited for one another)."""
+    import time
+
+    t = []
+    for k in (24, 256):
+        c = muca().Context([{"L": 8, "T": 1.4182, "n_walkers": 32}] * k, seed=3)
+        c.sweep_iter(50)
+        c.sync()
+        best = 1e9
+        for _ in range(5):
+            t0 = time.perf_counter()
+            c.sweep_iter(200)
+            c.sync()
+            best = min(best, time.perf_counter() - t0)
+        t.append(best)
+        c.close()
+    assert t[1] <= 4 * t[0], t
