@@ -48,6 +48,7 @@ struct GroupDev {
     uint32_t *spins;            // packed words, strides wstr (word) and cstr (walker)
     int64_t wstr, cstr;         // in words: (Wpad, 1), or (1, L * L * rw) walker by walker
     int rw;                     // words per row: Lw, or more walker by walker
+    int rows_seg;               // segments of a row of 33 to 48 sites (rows.cu)
     int32_t *tal;               // [3][Wpad]: E_J, E_Delta, M
     unsigned long long *hist;   // [nE]
     const uint32_t *thrE;       // the row of E_Delta = e_min in the table allocation
@@ -140,11 +141,13 @@ cudaError_t launch_sweeps_scan(int L, const GroupDev *groups_dev, const BlockDes
 // Site-per-lane launch (rows.cu), 3 <= L <= 64, with or without couplings per
 // bond: a walker's row is cut into seg segments of `lanes` consecutive sites,
 // one site per lane, and a block (one warp) serves per_warp = 32 / lanes
-// of its W walkers; seg = 0: not supported.
+// of its W walkers; seg = 0: not supported.  long_seg: the segments of rows of 33
+// to 48 sites, by the number of walkers that have such rows.
 struct RowShape {
     int seg, lanes, per_warp;
 };
-RowShape rows_shape(int L, int W);
+int rows_long_segments(int64_t walkers);
+RowShape rows_shape(int L, int long_seg);
 // Words per row of a lattice kept walker by walker.
 int rows_lattice_words(int L);
 // One launch sweeps up to kRowsMaxGroups groups of one kind (segments, row width

@@ -19,9 +19,9 @@
 // the latency of a row times the rows, not the arithmetic.  One site per lane
 // makes a row's latency independent of its length (up to 32 sites) and a
 // walker's bits warp-uniform; a chain kernel pays a dependent table load per
-// site instead.  Longer rows, and rows that would leave many lanes empty, are
-// cut into SEG segments of A lanes that follow one another (the segment
-// before is final), with 32 / A walkers side by side in a warp.
+// site instead.  Longer rows are cut into SEG segments of A lanes that follow one
+// another (the segment before is final); 32 / A walkers lie side by side in a
+// warp.
 //
 // Memory: the planes that a row reads lie in shared memory, rows at a fixed
 // pitch; behind the row being resolved, finished rows go back to the lattice
@@ -103,18 +103,6 @@ __device__ __forceinline__ void st_global_v4(void *a, uint4 v, bool p)
                  "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"((int)p)
                  : "memory");
 }
-// A spin of the lattice, read once by this lane: not kept in L1, which holds
-// the thresholds.
-__device__ __forceinline__ int ld_lattice(const char *p)
-{
-    int v;
-    asm volatile("ld.global.L1::no_allocate.s8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void prefetch_l2(const void *p, bool on)
-{
-    asm volatile("{.reg .pred q; setp.ne.s32 q, %1, 0; @q prefetch.global.L2 [%0];}" ::"l"(p), "r"((int)on));
-}
 __device__ __forceinline__ void cp4(void *smem, const void *gmem)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(shared_addr(smem)), "l"(gmem) : "memory");
@@ -129,22 +117,18 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 __device__ __forceinline__ void cp_wait_1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// How a walker's rows pass through shared memory, by the number of segments.
-//   planes: up to 12 sites all L; one to three segments the three planes that
-//     a row reads (z - 1, z, z + 1); four segments plane z alone, whose finished
-//     rows give way to those of plane z + 1, the z neighbours read from the
-//     lattice a step ahead;
+// How a walker's rows pass through shared memory:
+//   planes: up to 12 sites all L; else the three that a row reads (z - 1, z, z + 1);
 //   row L of a plane repeats row 0, the y + 1 neighbour of the last row, but for
 //     three segments, where a select takes its place;
 //   random words: two buffers for one or two segments, so that the next rows' words are
 //     stored as they are drawn; else one, the words waiting in registers.
-// The differences buy room: 48-site rows take 15.5 KB per warp, 14 warps per
-// SM, so that the benchmark's 2048 warps run in one wave (17.4 KB left 72 of
-// them to a second one: 157 -> 116 ms for 60 sweeps of 4096 walkers; with
-// plane z alone, the z neighbours' latency gave 146 ms).
+// The differences buy room: 48-site rows of three segments take 15.5 KB per warp, 14
+// warps per SM, so that the benchmark's 2048 warps run in one wave (17.4 KB left 72
+// of them to a second one: 157 -> 116 ms for 60 sweeps of 4096 walkers).
 // Rows are PITCH bytes apart, so a row's addresses are a register and a
 // constant.
-__host__ __device__ constexpr int rows_slots(int L, int seg) { return L <= 12 ? L : seg <= 3 ? 3 : 1; }
+__host__ __device__ constexpr int rows_slots(int L) { return L <= 12 ? L : 3; }
 __host__ __device__ constexpr bool rows_repeat0(int seg) { return seg != 3; }
 __host__ __device__ constexpr int rows_buffers(int seg) { return seg <= 2 ? 2 : 1; }
 // Words of a buffer: four rows touch at most L + 1 Philox blocks (rows that
@@ -156,7 +140,7 @@ __host__ __device__ constexpr int rows_random_words(int L) { return 4 * (L + 1);
 // slack.
 __host__ __device__ inline int rows_walker_words(int L, int seg, int per_warp, int pitch)
 {
-    const int rows = rows_slots(L, seg) * (L + rows_repeat0(seg)) + (seg <= 2 ? 2 : 0);
+    const int rows = rows_slots(L) * (L + rows_repeat0(seg)) + (seg <= 2 ? 2 : 0);
     const int n = rows_buffers(seg) * rows_random_words(L) + rows * (pitch / 4);
     const int want = per_warp <= 1 ? 0 : per_warp == 2 ? 16 : per_warp <= 4 ? 8 : 4;
     return want ? n + ((want - n) % 32 + 32) % 32 : (n + 3) / 4 * 4;
@@ -237,17 +221,14 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
     int8_t *const sp = reinterpret_cast<int8_t *>(mem + rows_buffers(SEG) * rows_random_words(L));
     constexpr bool REPEAT0 = rows_repeat0(SEG), TWO = rows_buffers(SEG) == 2;
     const int pb = (L + REPEAT0) * PITCH;  // bytes per plane
-    const bool ring = rows_slots(L, SEG) < L;
-    constexpr bool OWN = SEG > 3;  // plane z alone in shared memory
+    const bool ring = rows_slots(L) < L;
     const RowCopy<PITCH> copy{g.spins + (ptrdiff_t)w * g.cstr, g.wstr, L, g.Lw, g.rw, h};
     // a lattice whose rows lie as in shared memory is copied 16 bytes per lane
     const bool wide = g.wstr == 1 && g.rw * 4 == PITCH;
     char *const lat = reinterpret_cast<char *>(copy.g) + 16 * h;
     const uint32_t sp_a = shared_addr(sp);
     if (used) {
-        if (OWN) {
-            copy.plane_in(sp, 0, REPEAT0);
-        } else if (ring) {
+        if (ring) {
             copy.plane_in(sp, L - 1, REPEAT0);
             copy.plane_in(sp + pb, 0, REPEAT0);
             copy.plane_in(sp + 2 * pb, 1, REPEAT0);
@@ -272,14 +253,7 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
     int eo = (g.tal[g.Wpad + w] - g.e_min + kPad) * trow;
     int EJ = g.tal[w], Mg = g.tal[2 * g.Wpad + w];
     // byte offsets of planes z - 1, z, z + 1 in shared memory
-    int am = ring ? 0 : (L - 1) * pb, az = ring && !OWN ? pb : 0, ap = ring ? 2 * pb : pb;
-    // OWN: the lattice's bytes per row, the lanes' bytes of a row in it
-    const ptrdiff_t rsb = (ptrdiff_t)g.rw * g.wstr * 4;
-    const char *xg[SEG];
-#pragma unroll
-    for (int q = 0; q < SEG; ++q)
-        xg[q] = reinterpret_cast<const char *>(copy.g + (xo[q] >> 2) * g.wstr) + (xo[q] & 3);
-
+    int am = ring ? 0 : (L - 1) * pb, az = ring ? pb : 0, ap = ring ? 2 * pb : pb;
     // random words of the four rows from site `site` on: block b of the walker
     auto draw = [&](int site, int b, uint64_t sw) {
         return philox4x32_10(
@@ -303,8 +277,6 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
         for (int z = 0; z < L; ++z) {
             const uint2 *jrow = reinterpret_cast<const uint2 *>(g.J6) + z * L * L;
             const int dm = am - az, dp = ap - az;
-            const ptrdiff_t zm_o = (ptrdiff_t)(z ? z - 1 : L - 1) * L * rsb;
-            const ptrdiff_t zp_o = (ptrdiff_t)(z + 1 < L ? z + 1 : 0) * L * rsb;
             // per segment: the old spin of the next row to form, the new spin of
             // the row before the current one
             int own[SEG], ym[SEG];
@@ -327,8 +299,8 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                 uint4 drawn[SEG];
                 // The Site of row j, segment q, in two parts: the loads, and the
                 // rest.  x neighbours are the old spins (a step adds what the
-                // row changed), but for site L - 1 of a row of three or more
-                // segments, whose right neighbour, site 0, is final by then.
+                // row changed), but for site L - 1 of a row of three segments,
+                // whose right neighbour, site 0, is final by then.
                 struct Raw {
                     uint32_t rw;
                     int zm, zp, xl, xr, up;
@@ -342,14 +314,8 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                     const int8_t *const ru = SEG <= 2 || y0 + j + 1 < L ? row + (j + 1) * PITCH
                                              : sp + az + (REPEAT0 ? L * PITCH : 0);
                     r.rw = rnd[j * L + xo[q]];
-                    if (OWN) {
-                        const ptrdiff_t at = (ptrdiff_t)min(y0 + j, L - 1) * rsb;
-                        r.zm = ld_lattice(xg[q] + zm_o + at);
-                        r.zp = ld_lattice(xg[q] + zp_o + at);
-                    } else {
-                        r.zm = (rj + dm)[xo[q]];
-                        r.zp = (rj + dp)[xo[q]];
-                    }
+                    r.zm = (rj + dm)[xo[q]];
+                    r.zp = (rj + dp)[xo[q]];
                     r.xl = rj[xl_o[q]];
                     r.xr = rj[xr_o[q]];
                     r.up = ru[xo[q]];
@@ -454,15 +420,12 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                             dM += da;
                             s_new += da;
                             st_shared_u8(row_a + j * PITCH + xo[q], s_new, mine);
-                            if (j == 0 && REPEAT0 && !OWN)
+                            if (j == 0 && REPEAT0)
                                 st_shared_u8(row_a + L * PITCH + xo[q], s_new, mine && y0 == 0);
                             eo += trow * (__popc(acc & c.Pm & lanes) - __popc(acc & c.Mm & lanes));
                             if (SEG > 1 && q + 1 < SEG) edge = __shfl_sync(~0u, da, sbase + A - 1);
                             if (SEG == 2 && q == 0) first = __shfl_sync(~0u, da, sbase);
                         }
-                        // (plane z's row 0 gives way to plane z + 1's: its copy is made here)
-                        if (j == 0 && OWN)
-                            st_shared_u8(row_a + L * PITCH + xo[q], s_new, y0 == 0 && !idle[q]);
                         ym[q] = s_new;
                         c = n;
                     }
@@ -477,16 +440,8 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                 __syncwarp();
                 // the finished rows back to the lattice, and the same rows of plane
                 // z + 2 over those of plane z - 1
-                if (OWN && wide) {
-                    // the z + 1 rows, first touched by the steps above, eight rows
-                    // ahead from HBM into L2 (64 bytes per lane)
-                    const ptrdiff_t at = zp_o + (ptrdiff_t)(y0 + 8) * PITCH + 64 * h;
-                    prefetch_l2(reinterpret_cast<const char *>(copy.g) + at,
-                                used && 64 * h < 4 * PITCH && at < (ptrdiff_t)L * L * PITCH);
-                }
                 if (ring) {
-                    const int n = min(4, L - y0), zn = z + (OWN ? 1 : 2), z2 = zn < L ? zn : zn - L;
-                    const int dv = OWN ? 0 : dm;  // the rows that give way
+                    const int n = min(4, L - y0), z2 = z + 2 < L ? z + 2 : z + 2 - L;
                     if (wide) {
                         // n PITCH bytes, 16 per lane and turn
                         const ptrdiff_t o = (ptrdiff_t)(z * L + y0) * PITCH;
@@ -498,15 +453,15 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                             const uint4 v =
                                 *reinterpret_cast<const uint4 *>(row + (p ? 16 * h + at : 0));
                             st_global_v4(lat + o + at, v, p);
-                            cp16(row_a + dv + 16 * h + at, lat + i + at, p);
-                            if (t == 0 && REPEAT0 && !OWN)
-                                cp16(row_a + dv + L * PITCH + 16 * h, lat + i,
+                            cp16(row_a + dm + 16 * h + at, lat + i + at, p);
+                            if (t == 0 && REPEAT0)
+                                cp16(row_a + dm + L * PITCH + 16 * h, lat + i,
                                      used && y0 == 0 && 16 * h < PITCH);
                         }
                     } else if (used) {
                         copy.out(row, z, y0, n);
-                        copy.in(row + dv, z2, y0, n);
-                        if (REPEAT0 && !OWN && y0 == 0) copy.in(row + dv + L * PITCH, z2, 0, 1);
+                        copy.in(row + dm, z2, y0, n);
+                        if (REPEAT0 && y0 == 0) copy.in(row + dm + L * PITCH, z2, 0, 1);
                     }
                     cp_commit();
                     cp_wait_1();
@@ -519,11 +474,6 @@ __device__ __forceinline__ void rows_sweeps(const GroupDev &g, int A, int per_wa
                 }
             }
             // the next plane
-            if (OWN) {
-                cp_wait_all();  // its last rows came in just now
-                __syncwarp();
-                continue;
-            }
             const int t = am;
             am = az;
             az = ap;
@@ -609,17 +559,30 @@ sweep_rows_list_kernel(const __grid_constant__ RowsList list, uint32_t seed, uin
 
 }  // namespace
 
-// Segments and lanes of a row of L sites, for a group of W walkers.  Rows of up
-// to 32 sites are one segment.  Longer rows fill their warps best with three
-// segments of up to 16 lanes (L <= 48) or four, two walkers per warp; while the
-// walkers are fewer than the 608 schedulers, lanes are to spare and the time is
-// that of a row, so two segments and one walker per warp (L = 48: 608 walkers
-// on two segments 0.77 ms a sweep, 640 on three 1.34 ms).
-RowShape rows_shape(int L, int W)
+// Segments of rows of 33 to 48 sites, for all the walkers with such rows that are
+// swept together.  Two segments are one walker per warp; three, of up to 16
+// lanes, two walkers per warp, so half the warps, each slower (a step's passes
+// go on to the slower walker's last).  Two while the GPU holds all the walkers at
+// once (16 warps per SM); beyond that neither is ahead everywhere.
+// us per sweep, L = 48, T = 1, two and three segments:
+//   transition weights: 640 walkers 1398, 2521;  2048 1924, 3382;  4096 3699, 3963
+//   weights soon after a random start: 4096 walkers 2110, 1930
+// Rows of more than 48 sites are two segments, however many walkers there are (L = 64,
+// transition weights: 1024 walkers 3.46 ms a sweep, 4096 8.3; in four segments
+// 7.42 and 9.6).
+int rows_long_segments(int64_t walkers)
+{
+    int dev = 0, nsm = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        (void)cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return walkers <= (int64_t)16 * nsm ? 2 : 3;
+}
+
+RowShape rows_shape(int L, int long_seg)
 {
     RowShape s{0, 0, 0};
     if (L < 3 || L > 64) return s;
-    s.seg = L <= 32 ? 1 : W <= 608 ? 2 : L <= 48 ? 3 : 4;
+    s.seg = L <= 32 ? 1 : L <= 48 ? long_seg : 2;
     s.lanes = (L + s.seg - 1) / s.seg;
     s.per_warp = 32 / s.lanes;
     return s;
@@ -663,7 +626,7 @@ void launch(const GroupDev *const *g, const RowShape *sh, int n, size_t smem, ui
 
 int rows_kind(const GroupDev &g)
 {
-    return (rows_shape(g.L, g.W).seg * 100 + rows_pitch(g.L)) * 2 + (g.jmax > 0);
+    return (rows_shape(g.L, g.rows_seg).seg * 100 + rows_pitch(g.L)) * 2 + (g.jmax > 0);
 }
 
 cudaError_t launch_sweeps_rows(const GroupDev *const *g, int n, uint32_t seed, uint64_t sweep0,
@@ -675,7 +638,7 @@ cudaError_t launch_sweeps_rows(const GroupDev *const *g, int n, uint32_t seed, u
     size_t smem = 0;  // at most 16 KB: no opt-in
     const int kind = rows_kind(*g[0]);
     for (int i = 0; i < n; ++i) {
-        sh[i] = rows_shape(g[i]->L, g[i]->W);
+        sh[i] = rows_shape(g[i]->L, g[i]->rows_seg);
         if (sh[i].seg == 0 || rows_kind(*g[i]) != kind) return cudaErrorInvalidValue;
         smem = std::max(smem, rows_bytes_for(g[i]->L, sh[i]));
     }
@@ -693,7 +656,6 @@ cudaError_t launch_sweeps_rows(const GroupDev *const *g, int n, uint32_t seed, u
         MUCA_ROWS_LAUNCH(2, 48)
         MUCA_ROWS_LAUNCH(2, 64)
         MUCA_ROWS_LAUNCH(3, 48)
-        MUCA_ROWS_LAUNCH(4, 64)
 #undef MUCA_ROWS_LAUNCH
         default: return cudaErrorInvalidValue;
     }

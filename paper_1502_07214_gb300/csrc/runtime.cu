@@ -64,6 +64,7 @@ struct Group {
     int residency = MUCA_RES_GLOBAL;
     int wpb = 32;  // walkers per block
     int P = 1;     // lanes per walker
+    int rows_seg = 2;  // site-per-lane rows of 33 to 48 sites: segments
 };
 
 // Streams for the launches of one sweep call that run side by side.
@@ -360,6 +361,7 @@ GroupDev dev_of(const Group &g)
     d.wstr = g.by_walker ? 1 : g.Wpad;
     d.cstr = g.by_walker ? (int64_t)g.L * g.L * g.rw : 1;
     d.rw = g.rw;
+    d.rows_seg = g.rows_seg;
     d.tal = g.tal;
     d.hist = g.hist;
     d.thrE = g.thr ? g.thr + (size_t)(kPad + kGuard) * kRow : nullptr;
@@ -415,7 +417,7 @@ int upload_groups(muca_ctx *ctx)
 // Whether the site-per-lane kernel sweeps the group.
 bool on_rows(const Group &g)
 {
-    return rows_shape(g.L, g.W).seg > 0 && (g.jmax > 0 || g.residency == MUCA_RES_ROWS);
+    return rows_shape(g.L, g.rows_seg).seg > 0 && (g.jmax > 0 || g.residency == MUCA_RES_ROWS);
 }
 
 // Kernel kind of a group's block list (-1: none, the site-per-lane kernel).
@@ -454,6 +456,10 @@ int bonds_walkers_per_warp(int W)
 int build_blocks(muca_ctx *ctx)
 {
     std::vector<int> rows;
+    int64_t long_walkers = 0;
+    for (const Group &g : ctx->g)
+        if (on_rows(g) && g.L > 32 && g.L <= 48) long_walkers += g.W;
+    for (Group &g : ctx->g) g.rows_seg = rows_long_segments(long_walkers);
     std::vector<BlockDesc> b[kKinds];
     size_t sm[kKinds] = {};
     for (size_t gi = 0; gi < ctx->g.size(); ++gi) {
@@ -710,8 +716,6 @@ static int tune_group(muca_ctx *ctx, size_t gi, int residency, int wpb, int P)
     Group &g = ctx->g[gi];
     if (g.by_walker) {
         g.residency = MUCA_RES_ROWS;
-        g.wpb = rows_shape(g.L, g.W).per_warp;
-        g.P = rows_shape(g.L, g.W).lanes;
         return MUCA_OK;
     }
     const int smem_max = max_smem_per_block();
@@ -1063,7 +1067,7 @@ int muca_init(const muca_group *groups, int n_groups, const muca_options *opt, v
             g.beta = 1.0 / g.T;
             g.walker0 = w0 + (uint32_t)lo;
             g.by_walker = opt->residency == MUCA_RES_AUTO && opt->walkers_per_block == 0 &&
-                          opt->lanes_per_walker == 0 && rows_shape(g.L, g.W).seg > 0;
+                          opt->lanes_per_walker == 0 && rows_shape(g.L, g.rows_seg).seg > 0;
             w0 += (uint32_t)tot;
             g.lnW.assign(g.nE, 0.0);
             g.acc.assign((size_t)std::max(g.nE - 1, 1), 0.0);
@@ -1745,8 +1749,8 @@ int muca_get_config(muca_ctx *ctx, int group, int32_t *residency, int32_t *walke
     int rc = check_group_index(ctx, group);
     if (rc) return rc;
     const Group &g = ctx->g[group];
-    const RowShape rows = rows_shape(g.L, g.W);
-    const bool lane = g.jmax && on_rows(g);  // couplings on the site-per-lane kernel
+    const RowShape rows = rows_shape(g.L, g.rows_seg);
+    const bool lane = on_rows(g);
     if (residency) *residency = g.jmax ? MUCA_RES_BONDS : g.residency;
     if (walkers_per_block)
         *walkers_per_block = lane ? rows.per_warp : g.jmax ? bonds_walkers_per_warp(g.W) : g.wpb;

@@ -184,3 +184,19 @@ def test_many_small_groups_run_side_by_side():
         t.append(best)
         c.close()
     assert t[1] <= 4 * t[0], t
+
+
+@pytest.mark.parametrize("L,jj", [(33, None), (41, None), (48, None), (40, (1, 3)), (45, (-1, 2))])
+def test_three_segments_beyond_one_wave_of_warps(L, jj):
+    """Rows of 33 to 48 sites of more walkers than the GPU holds warps (16 per SM)
+    are cut into three segments, two walkers per warp; sampled walkers."""
+    V, W = L ** 3, 16 * torch.cuda.get_device_properties(0).multi_processor_count + 3
+    c = muca().Context([{"L": L, "T": 3.0, "n_walkers": n} for n in (W - 3, W)], seed=1)
+    assert [c.get_config(g)[2] for g in (0, 1)] == [(L + 2) // 3] * 2  # together
+    c.close()
+    c = muca().Context([{"L": L, "T": 3.0, "n_walkers": W - 3}], seed=1)
+    assert c.get_config(0)[1:] == (1, (L + 1) // 2)
+    c.close()
+    lnW = -1.5 * np.arange(V + 1) + wl.random_lnW(V + 1, L, scale=0.5)
+    run_against_oracle(L, 3.0, W, lnW, 2, walkers=[0, 1, 2, W // 2, W - 2, W - 1],
+                       bonds=None if jj is None else wl.random_bonds(L, jj[0], jj[1], seed=L))
