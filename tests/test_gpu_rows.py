@@ -200,3 +200,30 @@ def test_three_segments_beyond_one_wave_of_warps(L, jj):
     lnW = -1.5 * np.arange(V + 1) + wl.random_lnW(V + 1, L, scale=0.5)
     run_against_oracle(L, 3.0, W, lnW, 2, walkers=[0, 1, 2, W // 2, W - 2, W - 1],
                        bonds=None if jj is None else wl.random_bonds(L, jj[0], jj[1], seed=L))
+
+
+@pytest.mark.parametrize("L,W", [(5, 7), (12, 3), (13, 5), (16, 3), (20, 3), (32, 2), (34, 3),
+                                 (47, 2), (52, 2), (62, 2), (40, 2501)])
+def test_couplings_with_an_explicit_residency(L, W):
+    """A group whose lattice was laid out for another kernel (walker-minor words)
+    and then gets couplings: planes pass through shared memory word by word."""
+    V, n = L ** 3, 3
+    J = wl.random_bonds(L, -2, 3, seed=L)
+    lnW = -1.5 * np.arange(V + 1) + wl.random_lnW(V + 1, L, scale=0.5)
+    c = muca().Context([{"L": L, "T": 3.0, "n_walkers": W}], seed=L, residency=muca().RES_GLOBAL,
+                       walkers_per_block=32)
+    c.set_bonds(0, J)
+    c.set_lnW(0, lnW)
+    c.reserve_timeseries(n)
+    c.sweep_iter(n, record=True)
+    spins, tal = c.get_state(0)
+    ts = c.get_timeseries(0)
+    c.check_tallies()
+    c.close()
+    thr = oracle.build_table_bonds(L, 3.0, 3, 0, V, lnW)
+    for w in sorted({0, 1, W // 2, W - 1}):
+        sp = oracle.init_spins(L, L, w)
+        t = oracle.energies_bonds(L, sp, J).astype(np.int32)
+        ref = oracle.sweeps_bonds(L, J, 3, 0, V, thr, L, w, 0, n, sp, t, record=True)
+        assert np.array_equal(spins[w], sp) and np.array_equal(tal[w], t), w
+        assert np.array_equal(ts[:, :, w], ref), w
