@@ -75,7 +75,9 @@ typedef struct {
 } muca_group;
 
 /* Lattice residency of the sweep kernel. */
-#define MUCA_RES_AUTO 0   /* chosen by the autotuner (measured) */
+#define MUCA_RES_AUTO 0   /* MUCA_RES_ROWS for 3 <= L <= 64; for L = 2, or with a given
+                             walkers_per_block or lanes_per_walker, chosen by the
+                             autotuner (measured) */
 #define MUCA_RES_GLOBAL 1 /* spins stay in HBM/L2, site-major walker-minor */
 #define MUCA_RES_SMEM 2   /* each block keeps its walkers' lattices in shared memory */
 #define MUCA_RES_SPLIT 3  /* spins in HBM/L2; each block has one warp that runs the
@@ -94,9 +96,8 @@ typedef struct {
                              muca_options */
 #define MUCA_RES_ROWS 6   /* spins in HBM/L2, one lane per site of a row (or of a
                              segment of it), the row's decisions iterated together
-                             until they reproduce themselves (3 <= L <= 64): the
-                             choice of MUCA_RES_AUTO; reported by muca_get_config,
-                             not selectable in muca_options */
+                             until they reproduce themselves (3 <= L <= 64; other
+                             sizes as for MUCA_RES_AUTO) */
 
 /* debug_flags bits */
 #define MUCA_DEBUG_TALLY_CHECK 1 /* recompute E_J, E_Delta, M after every sweep call */
@@ -107,10 +108,13 @@ typedef struct {
     int32_t residency;         /* MUCA_RES_* */
     int32_t walkers_per_block; /* 0 = automatic; else 1 .. 32; a block is one warp, so
                                   walkers_per_block x lanes_per_walker <= 32 (== 32 for
-                                  global residency); fixed by L for MUCA_RES_SCAN */
+                                  global residency); fixed by L for MUCA_RES_SCAN,
+                                  by L and the context's walkers for MUCA_RES_ROWS
+                                  (0 .. 32 is accepted there, and not used) */
     int32_t lanes_per_walker;  /* 0 = automatic; else 1, 2, 4 or 8 threads serve one
                                   walker (they share its random numbers); fixed by L
-                                  (1 .. 16) for MUCA_RES_SCAN */
+                                  (1 .. 16) for MUCA_RES_SCAN, as walkers_per_block
+                                  for MUCA_RES_ROWS */
     int32_t shard_rank;        /* walker sharding over contexts (e.g. one per GPU):
                                   with shard_count = N > 1 the context holds shard
                                   shard_rank (0 .. N-1) of every group, walkers
@@ -452,9 +456,10 @@ int muca_set_state(muca_ctx *ctx, int group, const int8_t *spins);
  * running tallies: MUCA_OK or MUCA_ERR_TALLY_MISMATCH. */
 int muca_check_tallies(muca_ctx *ctx);
 
-/* Kernel configuration chosen for group g: residency (MUCA_RES_GLOBAL,
- * MUCA_RES_SMEM or MUCA_RES_SPLIT), walkers per block and lanes per walker
- * (0 for MUCA_RES_SPLIT).  Any output may be NULL. */
+/* Kernel configuration of group g: residency (MUCA_RES_*, MUCA_RES_BONDS for a
+ * group with couplings), walkers per block and lanes per walker (0 for
+ * MUCA_RES_SPLIT); of a group without couplings it can be given in muca_options
+ * again.  Any output may be NULL. */
 int muca_get_config(muca_ctx *ctx, int group, int32_t *residency, int32_t *walkers_per_block,
                     int32_t *lanes_per_walker);
 

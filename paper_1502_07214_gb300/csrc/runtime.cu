@@ -982,13 +982,16 @@ int muca_init(const muca_group *groups, int n_groups, const muca_options *opt, v
     *out = nullptr;
     if (!groups || n_groups < 1 || !opt)
         return fail(nullptr, MUCA_ERR_INVALID_ARG, "muca_init: need >= 1 group and options");
-    if (opt->residency < MUCA_RES_AUTO || opt->residency > MUCA_RES_SCAN)
+    const bool rows = opt->residency == MUCA_RES_ROWS;
+    if (!rows && (opt->residency < MUCA_RES_AUTO || opt->residency > MUCA_RES_SCAN))
         return fail(nullptr, MUCA_ERR_INVALID_ARG, "muca_init: bad residency %d", opt->residency);
     if (opt->walkers_per_block < 0 || opt->walkers_per_block > 32)
         return fail(nullptr, MUCA_ERR_INVALID_ARG, "muca_init: bad walkers_per_block %d",
                     opt->walkers_per_block);
-    if (opt->lanes_per_walker != 0 && opt->lanes_per_walker != 1 && opt->lanes_per_walker != 2 &&
-        opt->lanes_per_walker != 4 && opt->lanes_per_walker != 8 && opt->lanes_per_walker != 16)
+    if (rows ? opt->lanes_per_walker < 0 || opt->lanes_per_walker > 32
+             : opt->lanes_per_walker != 0 && opt->lanes_per_walker != 1 && opt->lanes_per_walker != 2 &&
+        opt->lanes_per_walker != 4 && opt->lanes_per_walker != 8 &&
+        opt->lanes_per_walker != 16)
         return fail(nullptr, MUCA_ERR_INVALID_ARG, "muca_init: bad lanes_per_walker %d",
                     opt->lanes_per_walker);
     const int shards = opt->shard_count > 1 ? opt->shard_count : 1;
@@ -1066,8 +1069,9 @@ int muca_init(const muca_group *groups, int n_groups, const muca_options *opt, v
             g.T = groups[i].T;
             g.beta = 1.0 / g.T;
             g.walker0 = w0 + (uint32_t)lo;
-            g.by_walker = opt->residency == MUCA_RES_AUTO && opt->walkers_per_block == 0 &&
-                          opt->lanes_per_walker == 0 && rows_shape(g.L, g.rows_seg).seg > 0;
+            g.by_walker = (rows || (opt->residency == MUCA_RES_AUTO && opt->walkers_per_block == 0 &&
+                                    opt->lanes_per_walker == 0)) &&
+                          rows_shape(g.L, g.rows_seg).seg > 0;
             w0 += (uint32_t)tot;
             g.lnW.assign(g.nE, 0.0);
             g.acc.assign((size_t)std::max(g.nE - 1, 1), 0.0);
@@ -1108,8 +1112,10 @@ int muca_init(const muca_group *groups, int n_groups, const muca_options *opt, v
                 if (ed[w] < g.e_min || ed[w] > g.e_max) g.in_window = false;
         }
         for (int i = 0; i < n_groups; ++i)
-            if ((rc = tune_group(ctx, i, opt->residency, opt->walkers_per_block,
-                                 opt->lanes_per_walker)) != MUCA_OK)
+            // (groups that the site-per-lane kernel does not take: another one's choice)
+            if ((rc = tune_group(ctx, i, rows ? MUCA_RES_AUTO : opt->residency,
+                                 rows ? 0 : opt->walkers_per_block,
+                                 rows ? 0 : opt->lanes_per_walker)) != MUCA_OK)
                 goto bad;
         if (n_groups > 1 && opt->residency == MUCA_RES_AUTO && opt->walkers_per_block == 0) {
             bool all_in = true;

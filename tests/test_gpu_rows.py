@@ -227,3 +227,26 @@ def test_couplings_with_an_explicit_residency(L, W):
         ref = oracle.sweeps_bonds(L, J, 3, 0, V, thr, L, w, 0, n, sp, t, record=True)
         assert np.array_equal(spins[w], sp) and np.array_equal(tal[w], t), w
         assert np.array_equal(ts[:, :, w], ref), w
+
+
+@pytest.mark.parametrize("L,W", [(2, 40), (3, 33), (8, 20), (22, 5), (48, 3), (64, 2)])
+def test_a_reported_configuration_can_be_given_again(L, W):
+    """A program that keeps get_config's result and pins it later."""
+    groups = [{"L": L, "T": 1.4182, "n_walkers": W}]
+    a = muca().Context(groups, seed=4)
+    cfg = a.get_config(0)
+    b = muca().Context(groups, seed=4, residency=cfg[0], walkers_per_block=cfg[1],
+                       lanes_per_walker=cfg[2])
+    assert b.get_config(0) == cfg
+    for c in (a, b):
+        c.run_graph(1, 4)
+    assert np.array_equal(a.get_state(0)[0], b.get_state(0)[0])
+    assert np.array_equal(a.get_lnW(0), b.get_lnW(0))
+    a.close()
+    b.close()
+    for bad in (muca().RES_BONDS, 7, -1):
+        with pytest.raises(muca().MucaError) as e:
+            muca().Context(groups, residency=bad)
+        assert e.value.code == muca().ERR_INVALID_ARG
+    with pytest.raises(muca().MucaError):
+        muca().Context(groups, residency=muca().RES_ROWS, lanes_per_walker=33)
