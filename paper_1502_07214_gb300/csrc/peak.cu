@@ -551,14 +551,17 @@ peak_kernel(PkBlocks bl, PkPlan p, int nE, double beta, double lo, double hi, in
     const int q = (int)cl.block_rank(), d = blockIdx.x / p.ncta;
     int slot = 0;
     // Exponents move by at most beta (hi - lo) |E - E'| in what is left of the
-    // interval: once that is 400 (the weights within e^+-400 of the reference) or
-    // less, the heaviest block is not looked for again
+    // interval: once that is 2, the heaviest block of the step before holds at least
+    // e^-2 of the weight that the heaviest has, and is not looked for again.  (At the
+    // ends of a wider interval it may hold next to nothing: the sums about it would
+    // be differences of large numbers, down to the sign of the third moment.)
+    // (Looked for in some seven steps of 63 instead of one: about 1.5 % of the kernel.)
     PkRef ref, peer;
     double z0;
     bool first = true;
     auto third_at = [&](double delta, double &cov) {
         double t;
-        const bool find = first || beta * (hi - lo) * nE > 400.0;
+        const bool find = first || beta * (hi - lo) * nE > 2.0;
         first = false;
         pk_moments<NT, SINGLE>(cl, part, slot, bl, p, d, nE, beta * delta, find, ref, peer, sh, shi,
                                cov, t, z0);

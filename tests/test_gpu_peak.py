@@ -245,3 +245,34 @@ def test_peak_of_a_series_that_fills_few_bins_of_a_wide_window(hw):
     assert abs(cs - want) <= 3e-14 * abs(want), abs(cs / want - 1)
     near = oracle.reweight_q(ej, ed, 0 * ed, lnW, 0, 1.0, V, [ds - 1e-4 * hw, ds + 1e-4 * hw])[:, 2]
     assert (near < want).all()
+
+
+@pytest.mark.parametrize("L,hw,n_jack", [(32, 1e-3, 0), (32, 1e-3, 200), (32, 3e-4, 200),
+                                         (64, 1e-4, 0), (64, 1e-4, 160)])
+def test_peak_between_two_states_from_pinned_ends(L, hw, n_jack):
+    """Two ground states and an interval at whose ends one of them holds all but
+    e^-40 .. e^-130 of the weight: the sign of dC/dDelta there must come from
+    sums about the state that holds it.  Closed form, as for the pin above."""
+    V, T = L ** 3, 0.25
+    beta = 1 / T
+    lnW = np.zeros(V + 1)
+    lnW[V] = -beta * 3 * V
+    ed = np.array([[V] * 3 + [0] * 5] * max(n_jack, 1), dtype=np.int32)
+    ds, _, cs, _, sub = muca().find_peak(dev(ed) * -3, dev(ed), lnW, 0, beta, 3 - hw, 3 + hw,
+                                         n_jack=n_jack)
+    want = 3 + np.log(3 / 5) / (beta * V), 3 * beta * V * float(V) / 4
+    assert abs(ds - want[0]) <= 1e-12 and abs(cs - want[1]) <= 1e-12 * want[1]
+    assert np.all(np.abs(sub[:, 0] - want[0]) <= 1e-12)
+    assert np.all(np.abs(sub[:, 1] - want[1]) <= 1e-12 * want[1])
+
+
+def test_peak_refuses_an_end_whose_weights_underflow():
+    """e^-13000 is zero in FP64: at the ends C and its slope are zero."""
+    V, T = 32 ** 3, 0.25
+    beta = 1 / T
+    lnW = np.zeros(V + 1)
+    lnW[V] = -beta * 3 * V
+    ed = np.array([[V] * 3 + [0] * 5] * 200, dtype=np.int32)
+    with pytest.raises(muca().MucaError) as e:
+        muca().find_peak(dev(ed) * -3, dev(ed), lnW, 0, beta, 2.9, 3.1, n_jack=200)
+    assert e.value.code == muca().ERR_INVALID_ARG
