@@ -365,7 +365,8 @@ int muca_reweight_noalloc(const int32_t *e_j, const int32_t *e_d, const int32_t 
  * MUCA_ERR_INVALID_ARG when [delta_lo, delta_hi] does not bracket the maximum
  * for the full series or a subset (dC/dDelta must be > 0 at delta_lo and < 0
  * at delta_hi); MUCA_ERR_WINDOW for a sample outside the window.  Its scratch
- * comes from muca_reweight's device memory pool; synchronises the stream. */
+ * comes from a device memory pool of which at most 256 MiB are kept between
+ * calls; synchronises the stream. */
 int muca_find_peak(const int32_t *e_j, const int32_t *e_d, int64_t n_rows, int32_t row_len,
                    int64_t row_stride, const double *lnW, int32_t e_min, int32_t n_e,
                    double beta, double delta_lo, double delta_hi, int32_t n_iter, int32_t n_jack,
@@ -388,7 +389,7 @@ int muca_find_peak(const int32_t *e_j, const int32_t *e_d, int64_t n_rows, int32
  *         minimum (full series), then (Delta_eqh, B) of each subset
  * MUCA_ERR_INVALID_ARG when the interval does not bracket Delta_eqh for the
  * full series or a subset; MUCA_ERR_WINDOW for a sample outside the window.
- * Its scratch comes from muca_reweight's device memory pool; synchronises the
+ * Its scratch comes from muca_find_peak's device memory pool; synchronises the
  * stream. */
 int muca_equal_height(const int32_t *e_d, int64_t n_rows, int32_t row_len, int64_t row_stride,
                       const double *lnW, int32_t e_min, int32_t n_e, double beta, int32_t split,

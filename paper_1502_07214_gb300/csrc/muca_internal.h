@@ -172,8 +172,9 @@ int max_smem_per_block();
 // Last-error text reported by muca_last_error(NULL) (thread-local).
 void set_last_error(const char *msg);
 
-// The device memory pool of the analysis calls' scratch (reweight.cu).
-int scratch_pool(cudaMemPool_t *out);
+// The device memory pools of the analysis calls' scratch (reweight.cu).
+enum class ScratchPool { reweight, peak };
+int scratch_pool(ScratchPool which, cudaMemPool_t *out);
 
 // Reweighting on caller-provided device scratch (reweight.cu).
 int reweight_check_args(const int32_t *e_j, const int32_t *e_d, const int32_t *m, int64_t n_rows,

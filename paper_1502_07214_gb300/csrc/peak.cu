@@ -939,7 +939,7 @@ extern "C" int muca_find_peak(const int32_t *e_j, const int32_t *e_d, int64_t n_
     const size_t b_w = al(pk_block_bytes(plan, n_sets));
     char *p = nullptr;
     cudaMemPool_t pool = nullptr;
-    const int rp = muca::scratch_pool(&pool);
+    const int rp = muca::scratch_pool(muca::ScratchPool::peak, &pool);
     if (rp != MUCA_OK) return rp;
     ce = cudaMallocFromPoolAsync((void **)&p, b_sums + b_sets + b_lnw + b_bnd + b_res + b_bad + b_w,
                                  pool, st);
@@ -1067,7 +1067,7 @@ extern "C" int muca_equal_height(const int32_t *e_d, int64_t n_rows, int32_t row
     const size_t b_bad = al((size_t)(n_sets + 1) * sizeof(int));
     char *p = nullptr;
     cudaMemPool_t pool = nullptr;
-    const int rp = muca::scratch_pool(&pool);
+    const int rp = muca::scratch_pool(muca::ScratchPool::peak, &pool);
     if (rp != MUCA_OK) return rp;
     cudaError_t ce = cudaMallocFromPoolAsync(
         (void **)&p, b_cnt + b_lnn + b_lnw + b_bnd + b_res + b_bad, pool, st);

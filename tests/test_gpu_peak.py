@@ -276,3 +276,21 @@ def test_peak_refuses_an_end_whose_weights_underflow():
     with pytest.raises(muca().MucaError) as e:
         muca().find_peak(dev(ed) * -3, dev(ed), lnW, 0, beta, 2.9, 3.1, n_jack=200)
     assert e.value.code == muca().ERR_INVALID_ARG
+
+
+def test_large_scratch_is_given_back():
+    """The scratch of 257 data sets of 262145 bins is 2.2 GB; the calls keep 256 MiB."""
+    V, T, w = 64 ** 3, 0.25, 256
+    beta = 1 / T
+    lnW = np.zeros(V + 1)
+    lnW[V] = -beta * 3 * V
+    ed = dev(np.array([[V] * 3 + [0] * 5] * w, dtype=np.int32))
+    ej = -3 * ed
+    muca().find_peak(ej, ed, lnW, 0, beta, 2.9999, 3.0001)
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    ds, _, cs, _, _ = muca().find_peak(ej, ed, lnW, 0, beta, 2.9999, 3.0001, n_jack=w)
+    assert abs(ds - (3 + np.log(3 / 5) / (beta * V))) <= 1e-12
+    assert abs(cs - 3 * beta * V * float(V) / 4) <= 1e-12 * cs
+    muca().equal_height(ed, lnW, 0, beta, V // 2, 2.9999, 3.0001, n_jack=w)
+    assert free0 - torch.cuda.mem_get_info()[0] <= 300 << 20
