@@ -36,8 +36,8 @@ inline size_t table_rows(int nE) { return (size_t)nE + 2 * (kGuard + kPad); }
 // the site-per-lane kernel sweeps (rows.cu) keep the same words walker by
 // walker instead, word (row, j) of walker w at
 //   spins[w * L * L * rw + row * rw + j],
-// rows of rw >= Lw words (the words past Lw are 0), so that the lanes of a row
-// read consecutive bytes.  Either way word (row, j) of walker w is
+// rows of rw >= Lw words (the words past Lw are not used and hold anything), so
+// that the lanes of a row read consecutive bytes.  Either way word (row, j) of walker w is
 //   spins[(row * rw + j) * wstr + w * cstr].
 
 // Per-group parameters in device memory.
@@ -148,7 +148,7 @@ struct RowShape {
 };
 int rows_long_segments(int64_t walkers);
 RowShape rows_shape(int L, int long_seg);
-// Words per row of a lattice kept walker by walker.
+// Words per row of a lattice kept walker by walker with padded rows.
 int rows_lattice_words(int L);
 // One launch sweeps up to kRowsMaxGroups groups of one kind (segments, row width
 // in shared memory, couplings or not).

@@ -994,6 +994,12 @@ int muca_init(const muca_group *groups, int n_groups, const muca_options *opt, v
         opt->lanes_per_walker != 16)
         return fail(nullptr, MUCA_ERR_INVALID_ARG, "muca_init: bad lanes_per_walker %d",
                     opt->lanes_per_walker);
+    // the groups that the site-per-lane kernel takes, for their sizes
+    auto lane_per_site = [&](int L) {
+        return (rows || (opt->residency == MUCA_RES_AUTO && opt->walkers_per_block == 0 &&
+                         opt->lanes_per_walker == 0)) &&
+               rows_shape(L, 2).seg > 0;
+    };
     const int shards = opt->shard_count > 1 ? opt->shard_count : 1;
     const int srank = opt->shard_count > 1 ? opt->shard_rank : 0;
     if (opt->shard_count < 0 || opt->shard_rank < 0 || (opt->shard_count <= 1 && opt->shard_rank) ||
@@ -1046,6 +1052,18 @@ int muca_init(const muca_group *groups, int n_groups, const muca_options *opt, v
         CKI(cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming));
         CKI(cudaMalloc(&ctx->d_err, sizeof(int)));
         CKI(cudaMalloc(&ctx->d_groups, n_groups * sizeof(GroupDev)));
+        // Rows of the site-per-lane lattices are padded to the kernel's row width in
+        // shared memory, for 16-byte copies, while the padding of all groups takes at
+        // most a sixteenth of the free memory; else they are packed, and the kernel
+        // copies words.  (Padded rows are up to 1.6 times as long.  us per sweep of
+        // 4096 walkers, padded and packed: L = 20 238, 340; L = 36 1317, 1532.)
+        size_t pad = 0, free_b = 0, all_b = 0;
+        for (int i = 0; i < n_groups; ++i)
+            if (lane_per_site(groups[i].L))
+                pad += (size_t)groups[i].n_walkers / shards * groups[i].L * groups[i].L *
+                       (rows_lattice_words(groups[i].L) - (groups[i].L + 3) / 4) * sizeof(uint32_t);
+        CKI(cudaMemGetInfo(&free_b, &all_b));
+        const bool padded = pad <= free_b / 16;
         uint32_t w0 = 0;
         ctx->g.resize(n_groups);
         for (int i = 0; i < n_groups; ++i) {
@@ -1069,22 +1087,13 @@ int muca_init(const muca_group *groups, int n_groups, const muca_options *opt, v
             g.T = groups[i].T;
             g.beta = 1.0 / g.T;
             g.walker0 = w0 + (uint32_t)lo;
-            g.by_walker = (rows || (opt->residency == MUCA_RES_AUTO && opt->walkers_per_block == 0 &&
-                                    opt->lanes_per_walker == 0)) &&
-                          rows_shape(g.L, g.rows_seg).seg > 0;
+            g.by_walker = lane_per_site(g.L);
             w0 += (uint32_t)tot;
             g.lnW.assign(g.nE, 0.0);
             g.acc.assign((size_t)std::max(g.nE - 1, 1), 0.0);
-            g.rw = g.by_walker ? rows_lattice_words(g.L) : g.Lw;
-            if (g.by_walker && cudaMalloc(&g.spins, lattice_words(g) * sizeof(uint32_t)) != cudaSuccess) {
-                // no room for padded rows: the walker-minor layout and its kernels
-                (void)cudaGetLastError();
-                g.spins = nullptr;
-                g.by_walker = false;
-                g.rw = g.Lw;
-            }
+            g.rw = g.by_walker && padded ? rows_lattice_words(g.L) : g.Lw;
             const size_t sbytes = lattice_words(g) * sizeof(uint32_t);
-            if (!g.spins) CKI(cudaMalloc(&g.spins, sbytes));
+            CKI(cudaMalloc(&g.spins, sbytes));
             CKI(cudaMemsetAsync(g.spins, 0, sbytes, ctx->stream));
             CKI(cudaMalloc(&g.tal, (size_t)3 * g.Wpad * sizeof(int32_t)));
             CKI(cudaMemsetAsync(g.tal, 0, (size_t)3 * g.Wpad * sizeof(int32_t), ctx->stream));

@@ -250,3 +250,38 @@ def test_a_reported_configuration_can_be_given_again(L, W):
         assert e.value.code == muca().ERR_INVALID_ARG
     with pytest.raises(muca().MucaError):
         muca().Context(groups, residency=muca().RES_ROWS, lanes_per_walker=33)
+
+
+def test_lattices_that_fit_only_with_packed_rows():
+    """Groups whose lattices fit the free memory with packed rows, not with rows
+    padded for 16-byte copies, are accepted, and swept in that layout."""
+    Ls = [17, 13, 22, 34, 50] + [17] * 8
+    groups = [{"L": L, "T": 3.0, "n_walkers": 10000 if i > 4 else 3} for i, L in enumerate(Ls)]
+    packed = sum(s["n_walkers"] * s["L"] ** 2 * ((s["L"] + 3) // 4) * 4 for s in groups)
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    ballast = torch.empty(torch.cuda.mem_get_info()[0] - packed - (100 << 20), dtype=torch.uint8,
+                          device="cuda")
+    try:
+        c = muca().Context(groups, seed=6)
+        out = []
+        for g, s in enumerate(groups):
+            assert c.get_config(g)[0] == muca().RES_ROWS
+            V = s["L"] ** 3
+            c.set_lnW(g, -1.5 * np.arange(V + 1) + wl.random_lnW(V + 1, g, scale=0.5))
+        c.sweep_iter(2)
+        for g in range(6):
+            out.append((c.get_state(g), c.get_lnW(g), c.specs[g]["first_walker"]))
+        c.check_tallies()
+        c.close()
+    finally:
+        del ballast
+        torch.cuda.empty_cache()
+    for s, ((spins, tal), lnW, w0) in zip(groups, out):
+        L, V = s["L"], s["L"] ** 3
+        thr = oracle.build_table(L, 3.0, 0, V, lnW)
+        for w in (0, 1, len(spins) - 1):
+            sp = oracle.init_spins(L, 6, w0 + w)
+            t = oracle.energies(L, sp).astype(np.int32)
+            oracle.sweeps(L, 0, V, thr, 6, w0 + w, 0, 2, sp, t)
+            assert np.array_equal(spins[w], sp) and np.array_equal(tal[w], t), (L, w)
