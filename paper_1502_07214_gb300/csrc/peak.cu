@@ -25,6 +25,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <string>
@@ -672,9 +673,11 @@ struct EqLive {
 
 // The two peak bins at beta Delta = bd among bins [e0, e1) (relative to e_min,
 // -1 when a side is empty); reach: beta times the width of the interval that
-// holds every field still to come, bd among them.
+// holds every field still to come, bd among them; slack: above the rounding of
+// the values that are compared.
 __device__ void eqh_peaks(const double *lnn, const double *lnW, int e0, int e1, int e_min,
-                          int split, double bd, double reach, EqLive &live, int (&p)[2],
+                          int split, double bd, double reach, double slack, EqLive &live,
+                          int (&p)[2],
                           double (&v)[2], double *sh, int *shi)
 {
     v[0] = v[1] = -INFINITY;
@@ -694,8 +697,7 @@ __device__ void eqh_peaks(const double *lnn, const double *lnW, int e0, int e1, 
         }
         const double w = eqh_lnp(n, bd, e_min + e, lnW[e]);
         const int s = e_min + e < split ? 0 : 1;
-        // a thousandth covers the rounding of both sides
-        if (live.have && (w - top[s]) + reach * (double)abs(e - live.p[s]) < -1e-3) {
+        if (live.have && (w - top[s]) + reach * (double)abs(e - live.p[s]) < -slack) {
             live.mask &= ~bit;
             continue;
         }
@@ -746,7 +748,8 @@ __device__ double eqh_cluster_peaks(cg::cluster_group &cl, EqPart *part, int &sl
 // bisection on g = ln P_low - ln P_high, then the barrier at Delta_eqh.
 __global__ void __launch_bounds__(kPkThreads)
 eqh_kernel(const double *__restrict__ lnn_all, const double *__restrict__ lnW, int nE, int e_min,
-           int split, double beta, double lo, double hi, int n_iter, double *res, int *bad)
+           int split, double beta, double lo, double hi, int n_iter, double slack, double *res,
+           int *bad)
 {
     __shared__ double sh[64];
     __shared__ int shi[64];
@@ -761,7 +764,8 @@ eqh_kernel(const double *__restrict__ lnn_all, const double *__restrict__ lnW, i
     auto peaks = [&](double bd, int &pl, int &pr, double &vl, double &vr) {
         double v[2];
         int p[2];
-        eqh_peaks(lnn, lnW, e0, e1, e_min, split, bd, beta * (hi - lo), live, p, v, sh, shi);
+        eqh_peaks(lnn, lnW, e0, e1, e_min, split, bd, beta * (hi - lo), slack, live, p, v, sh,
+                  shi);
         vl = v[0];
         vr = v[1];
         pl = p[0];
@@ -1051,9 +1055,17 @@ extern "C" int muca_equal_height(const int32_t *e_d, int64_t n_rows, int32_t row
         !std::isfinite(delta_hi) || !(delta_lo < delta_hi))
         return pk_fail(MUCA_ERR_INVALID_ARG,
                        "muca_equal_height: need beta > 0 and delta_lo < delta_hi");
-    for (int e = 0; e < n_e; ++e)
+    double lnw_max = 0.0;
+    for (int e = 0; e < n_e; ++e) {
         if (!std::isfinite(lnW[e]))
             return pk_fail(MUCA_ERR_INVALID_ARG, "muca_equal_height: lnW not finite");
+        lnw_max = std::max(lnw_max, std::fabs(lnW[e]));
+    }
+    // ln P and its prediction from the step before are some ten operations on
+    // numbers of this size, of at most half a unit in the last place (2^-53) each
+    const double e_max = std::max(std::fabs((double)e_min), std::fabs((double)e_min + n_e));
+    const double slack =
+        1e-3 + 0x1p-48 * (beta * std::max(std::fabs(delta_lo), std::fabs(delta_hi)) * e_max + lnw_max);
     cudaStream_t st = (cudaStream_t)stream;
     const int n_blocks = n_jack > 0 ? n_jack : 1, n_sets = 1 + n_jack;
     std::vector<int64_t> bnd(n_blocks + 1);
@@ -1109,7 +1121,7 @@ extern "C" int muca_equal_height(const int32_t *e_d, int64_t n_rows, int32_t row
         PCK(cluster_config((const void *)eqh_kernel, n_sets, kPkThreads, 8, st, cfg, attr));
         PCK(cudaLaunchKernelEx(&cfg, eqh_kernel, (const double *)lnn, (const double *)d_lnW,
                                (int)n_e, (int)e_min, (int)split, beta, delta_lo, delta_hi,
-                               (int)n_iter, d_res, d_bad + 1));
+                               (int)n_iter, slack, d_res, d_bad + 1));
     }
     PCK(cudaMemcpyAsync(res.data(), d_res, res.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
     PCK(cudaMemcpyAsync(bad.data(), d_bad, bad.size() * sizeof(int), cudaMemcpyDeviceToHost, st));

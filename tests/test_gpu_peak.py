@@ -294,3 +294,19 @@ def test_large_scratch_is_given_back():
     assert abs(cs - 3 * beta * V * float(V) / 4) <= 1e-12 * cs
     muca().equal_height(ed, lnW, 0, beta, V // 2, 2.9999, 3.0001, n_jack=w)
     assert free0 - torch.cuda.mem_get_info()[0] <= 300 << 20
+
+
+@pytest.mark.parametrize("L,hw", [(4, 1e10), (16, 1e8), (16, 1e10), (64, 1e6), (64, 1e8), (64, 1e10)])
+def test_equal_height_from_a_very_wide_interval(L, hw):
+    """The search drops bins that cannot become a peak any more; at wide fields
+    ln P is some 1e13 and rounds to more than a thousandth, so the bound has to
+    grow with it.  Two states: n1 / n0 samples, closed form; the bisection's 60
+    steps leave 2 hw 2^-60, the fields of the last ones round like Delta V."""
+    V, T = L ** 3, 0.25
+    beta = 1 / T
+    lnW = np.zeros(V + 1)
+    lnW[V] = -beta * 3 * V
+    ed = np.array([[V] * 3 + [0] * 5] * 40, dtype=np.int32)
+    got = muca().equal_height(dev(ed), lnW, 0, beta, V // 2, 3 - 0.7 * hw, 3 + hw)
+    assert abs(got[0] - (3 + np.log(3 / 5) / (beta * V))) <= 2 * hw * 2.0 ** -60 + 1e-12
+    assert got[4][:2] == (0, V)
