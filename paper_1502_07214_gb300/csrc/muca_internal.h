@@ -80,6 +80,10 @@ struct BlockDesc {
 
 // Launch helpers implemented in sweep.cu.  All return a cudaError_t.
 cudaError_t launch_init_spins(const GroupDev &g, uint32_t seed, cudaStream_t st);
+// Words v0 .. v0 + nv - 1 (row Lw + j) of a lattice kept walker by walker, to or from
+// walker-minor order [nv][Wpad].
+cudaError_t launch_walker_minor(const GroupDev &g, uint32_t *minor, int v0, int nv, bool to_minor,
+                                cudaStream_t st);
 // mode 0: write the recomputed tallies; mode 1: compare and raise *err on mismatch.
 cudaError_t launch_energies(const GroupDev &g, int mode, int *err, cudaStream_t st);
 // One launch sweeping every block of `blocks` (n_blocks of them) with
