@@ -305,7 +305,9 @@ int muca_iterate(muca_ctx *ctx, int32_t max_iters, int32_t sweeps_per_iter, doub
  *                 must satisfy e_min <= E_Delta < e_min + n_e
  *   beta, V       inverse temperature and number of sites
  *   delta_grid    host FP64 [n_grid]
- *   precision     64: FP64 arithmetic; 32: FP32 arithmetic (max-shifted
+ *   precision     64: FP64 arithmetic (the sums of narrow grids are polynomials in
+ *                 the field about the grid's middle, so a field's last bits
+ *                 depend on the grid's ends); 32: FP32 arithmetic (max-shifted
  *                 exponents carried as float pairs, Kahan-compensated sums)
  *   out           host FP64 [n_grid][5]: <E_J>, <E_Delta>, C,
  *                 chi = beta V (<m^2> - <|m|>^2), U4 = 1 - <m^4> / (3 <m^2>^2),
