@@ -54,18 +54,21 @@ def env_int(k, d):
 
 # DRAM bytes (read + write) per sweep of the benchmark workload, from one ncu
 # capture of each kernel in this configuration (a launch of 2 sweeps after
-# three 1000-sweep weight iterations): split kernel 926.8 MB read + 848.5 MB
-# written, row-scan kernel 1943.5 MB read + 881.9 MB written.  Valid only for
-# the kernel source the counters were taken on; empty (traffic reported as
-# null) while no capture of the current source exists.
+# three 1000-sweep weight iterations; of the site-per-lane kernel after 60
+# sweeps): split kernel 926.8 MB read + 848.5 MB written, row-scan kernel
+# 1943.5 MB read + 881.9 MB written, site-per-lane kernel 934.8 MB read + 850.8
+# MB written.  Valid only for the kernel source the counters were taken on;
+# empty (traffic reported as null) while no capture of the current source exists.
 TRAFFIC_PER_SWEEP = {3: (926.811392e6 + 848.504064e6) / 2,
-                     4: (1943.472e6 + 881.874176e6) / 2}
+                     4: (1943.472e6 + 881.874176e6) / 2,
+                     6: (934.84928e6 + 850.848256e6) / 2}
 
 
 # L2 bytes (32-byte sectors through the L2, lts__t_sectors.sum) per sweep from
-# the same captures: split kernel 216.3 M sectors, row-scan kernel 338.3 M
-# sectors per 2-sweep launch.  Same validity rule as the DRAM traffic.
-L2_PER_SWEEP = {3: 216.3e6 * 32 / 2, 4: 338.261052e6 * 32 / 2}
+# the same captures: split kernel 216.3 M sectors, row-scan kernel 338.3 M,
+# site-per-lane kernel 161.3 M sectors per 2-sweep launch.  Same validity rule
+# as the DRAM traffic.
+L2_PER_SWEEP = {3: 216.3e6 * 32 / 2, 4: 338.261052e6 * 32 / 2, 6: 161.31854e6 * 32 / 2}
 
 PROBE_KINDS = {0: "IMAD a=a*a+b", 1: "IADD3 a=a+b+c", 2: "LOP3 a=(a&b)^c",
                3: "half IMAD, half IADD3"}
@@ -735,8 +738,7 @@ def main():
                     help="sweep kernel configuration of --profile sweep")
     ap.add_argument("--sweep-config", default="",
                     help="residency,walkers per block,lanes per walker of the benchmark's "
-                         "context instead of the autotuner's choice (for profiler runs, whose "
-                         "serialised launches change the autotuner's timings)")
+                         "context instead of the default's (e.g. 3,16,0: the split kernel)")
     args = ap.parse_args()
     if args.profile == "probes":
         # the device probes alone, printed as JSON (short runs for a capture)
