@@ -42,9 +42,9 @@
 // (sweep.cu's split kernel for L = 8 .. 32, scan.cu's for L = 48, one thread
 // per walker for L % 4 != 0 and for couplings), time per call:
 //   L = 8, T = 2, 64 walkers, 200 sweeps and merge    11.8 -> 4.4 ms
-//   L = 16, T = 1, 1024 walkers, 500 sweeps and merge 94.8 -> 24.6 ms
+//   L = 16, T = 1, 1024 walkers, 500 sweeps and merge 94.8 -> 25.0 ms
 //   L = 32, T = 0.9, 2048 walkers, 150 and merge      157 -> 43.4 ms
-//   L = 8 .. 32 in one context, 12288 walkers, 60     112 -> 43.5 ms
+//   L = 8 .. 32 in one context, 12288 walkers, 60     112 -> 42.2 ms
 //   L = 22, T = 1.4182, 1000 walkers, 50 and merge    76.9 -> 6.8 ms
 //   L = 28, T = 1, 1024 walkers, 100 recorded         74.4 -> 26.0 ms
 //   L = 48, T = 0.9, 4096 walkers, 60 recorded        248 -> 115 ms
