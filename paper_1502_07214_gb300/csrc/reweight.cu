@@ -757,89 +757,110 @@ grid_kernel_f32(BinStats<float> s, int nE, int e_min, float beta, int V,
     }
 }
 
+constexpr int kStats = 8;
+
+// Sums of K values over the block (of NW warps if given); every thread gets them.
+template <int K, int NW = 0>
+__device__ __forceinline__ void block_sum_plain(double (&v)[K], double *sh)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = NW ? NW : blockDim.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
+    __syncthreads();
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < K; ++k) sh[wid * K + k] = v[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        double a = sh[k];
+        for (int i = 1; i < nw; ++i) a += sh[i * K + k];
+        v[k] = a;
+    }
+}
+
+// C, chi and the means of one field from its sums T about the reference bin's or
+// block's (E0, J0, M0): weight, E, E_J, |m|, m^2, m^4, (E_J - J0)(E - E0), the
+// variance of |m| about M0.
+__device__ __forceinline__ void put_field(const double (&T)[kStats], int E0, double J0, double M0,
+                                          double beta, int V, double *o)
+{
+    const double Z = T[0], mE = T[1] / Z, mJ = T[2] / Z, mu = T[3] / Z;
+    const double m2 = T[4] / Z, m4 = T[5] / Z;
+    o[0] = J0 + mJ;
+    o[1] = (double)E0 + mE;
+    o[2] = -beta * (T[6] / Z - mE * mJ);
+    o[3] = beta * (double)V * (T[7] / Z - mu * mu);
+    o[4] = 1.0 - m4 / (3.0 * m2 * m2);
+}
+
 // ------------------------------------------- FP64 stage B, bin by bin
-// Grids that are too wide for blocks of bins (below): every field visits every
-// occupied bin, the sums are compensated, C and chi are taken in a second pass
-// about the means.
-// Exponent of Eq. 3: a = -(c E) - lnW(E), c = beta Delta_k.  It is used to
-// find the bin E* of the largest weight; the normalised exponents are then
-// formed as -c (E - E*) - (lnW(E) - lnW(E*)) so that two O(beta Delta V) numbers
-// are never subtracted.
-__device__ __forceinline__ double expo64(double c, int E, double lw)
-{
-    return __dsub_rn(-__dmul_rn(c, (double)E), lw);
-}
-
-__device__ __forceinline__ double rel64(double c, int dE, double lw, double lstar)
-{
-    return __dsub_rn(-__dmul_rn(c, (double)dE), __dsub_rn(lw, lstar));
-}
-
-__global__ void __launch_bounds__(256)
+// Grids that are too wide for blocks of bins (below), one field per CTA.  The
+// sums are taken about the field's heaviest bin (to the precision of an FP32
+// logarithm of its samples: any bin near it serves), which holds at least
+// 1 / n_e of the weight or so; so one pass gives the centred sums too.
+// Exponents are formed as -c (E - E0) - (lnW(E) - lnW(E0)), c = beta Delta_k,
+// so that two O(beta Delta V) numbers are never subtracted.  Each thread adds up
+// 32 bins at a time, and those sums.
+//   4096 fields, beta = 0.7, half width 1, 6.4e5 samples: 4097 bins 1.47 ms a call,
+//   32769 bins 5.0, 262145 bins 29.4 (three passes of compensated sums: 3.6, 8.9,
+//   41.1; polynomials over blocks of one bin: 2.1, 15.1, 102)
+__global__ void __launch_bounds__(512)
 grid_kernel_f64(BinStats<double> s, int nE, int e_min, double beta, int V,
                 const double *__restrict__ cgrid, double *__restrict__ out)
 {
-    __shared__ double sh[64];
+    __shared__ double shv[32];
     __shared__ int she[32];
-    const int k = blockIdx.x;
-    const double c = cgrid[k];
-    double amax = -INFINITY;
-    int estar = 0x7FFFFFFF;
-    for (int e = threadIdx.x; e < nE; e += blockDim.x)
-        if (s.n[e] > 0) {
-            const double a = expo64(c, e_min + e, s.lw[e]);
-            if (a > amax) {
-                amax = a;
-                estar = e;
+    __shared__ double sh[16 * kStats];
+    const double c = cgrid[blockIdx.x];
+    double best = -INFINITY;
+    int at = 0x7FFFFFFF;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < nE; e += blockDim.x) {
+        const double n = s.n[e], lw = s.lw[e];
+        if (n > 0.0) {
+            const double a = (-(c * (double)(e_min + e)) - lw) + (double)__logf((float)n);
+            if (a > best) {
+                best = a;
+                at = e;
             }
         }
-    block_argmax(amax, estar, sh, she);
-    const double lstar = s.lw[estar];
-    KSum<double> acc[6];
+    }
+    block_argmax(best, at, shv, she);
+    if (at >= nE) at = 0;  // no sample lies in the window (the call fails)
+    const double l0 = s.lw[at], J0 = s.mej[at], M0 = s.cm[at];
+    double T[kStats];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) acc[i].init();
-    for (int e = threadIdx.x; e < nE; e += blockDim.x) {
-        const double n = s.n[e];
-        if (n <= 0) continue;
-        const double d = rel64(c, e - estar, s.lw[e], lstar);
-        if (d < -800.0) continue;
-        const double w = exp(d);
-        const double wn = w * n;
-        acc[0].add(wn);
-        acc[1].add(wn * (double)(e_min + e));
-        acc[2].add(wn * s.mej[e]);
-        acc[3].add(wn * s.cm[e]);
-        acc[4].add(w * s.q2[e]);
-        acc[5].add(w * s.q4[e]);
+    for (int j = 0; j < kStats; ++j) T[j] = 0.0;
+    for (int e0 = threadIdx.x; e0 < nE; e0 += 32 * blockDim.x) {
+        double S[kStats];
+#pragma unroll
+        for (int j = 0; j < kStats; ++j) S[j] = 0.0;
+        const int e1 = min(nE, e0 + 32 * (int)blockDim.x);
+#pragma unroll 4
+        for (int e = e0; e < e1; e += blockDim.x) {
+            const double n = s.n[e], lw = s.lw[e];
+            if (!(n > 0.0)) continue;
+            const double dE = (double)(e - at), d = __dsub_rn(-__dmul_rn(c, dE), __dsub_rn(lw, l0));
+            if (d < -800.0) continue;
+            const double w = exp(d), wn = w * n;
+            const double dJ = s.mej[e] - J0, dM = s.cm[e] - M0, wj = wn * dJ, wm = wn * dM;
+            S[0] += wn;
+            S[1] = fma(wn, dE, S[1]);
+            S[2] += wj;
+            S[3] += wm;
+            S[4] = fma(w, s.q2[e], S[4]);
+            S[5] = fma(w, s.q4[e], S[5]);
+            S[6] = fma(wj, dE, S[6]);
+            S[7] += fma(w, s.vb[e], wm * dM);
+        }
+#pragma unroll
+        for (int j = 0; j < kStats; ++j) T[j] += S[j];
     }
-    double S[6];
-    block_sum<double, 6>(acc, S, sh);
-    const double Z = S[0], mE = S[1] / Z, mJ = S[2] / Z, mu = S[3] / Z;
-    KSum<double> acc2[2];
-    acc2[0].init();
-    acc2[1].init();
-    for (int e = threadIdx.x; e < nE; e += blockDim.x) {
-        const double n = s.n[e];
-        if (n <= 0) continue;
-        const double d = rel64(c, e - estar, s.lw[e], lstar);
-        if (d < -800.0) continue;
-        const double w = exp(d);
-        const double wn = w * n;
-        acc2[0].add(wn * ((s.mej[e] - mJ) * ((double)(e_min + e) - mE)));
-        const double dm = s.cm[e] - mu;
-        acc2[1].add(w * s.vb[e] + wn * (dm * dm));
-    }
-    double S2[2];
-    block_sum<double, 2>(acc2, S2, sh);
-    if (threadIdx.x == 0) {
-        double *o = out + 5 * (int64_t)k;
-        o[0] = mJ;
-        o[1] = mE;
-        o[2] = -beta * (S2[0] / Z);
-        o[3] = beta * (double)V * (S2[1] / Z);
-        const double m2 = S[4] / Z, m4 = S[5] / Z;
-        o[4] = 1.0 - m4 / (3.0 * m2 * m2);
-    }
+    block_sum_plain<kStats>(T, sh);
+    if (threadIdx.x == 0) put_field(T, e_min + at, J0, M0, beta, V, out + 5 * (int64_t)blockIdx.x);
 }
 
 // ------------------------------------------- FP64 stage B, blocks of bins
@@ -874,7 +895,6 @@ grid_kernel_f64(BinStats<double> s, int nE, int e_min, double beta, int V,
 // a block's reference bin cost the covariance of a narrow distribution a
 // decimal digit that FP32 does not have to spare (3e-5 to 5e-5 where 1e-5 is
 // asked, on a rough 262145-bin window).
-constexpr int kStats = 8;
 constexpr int kDegMax = 20;
 constexpr int kRgThreads = 128;
 constexpr double kXMax = 1.2;
@@ -887,18 +907,16 @@ struct BlockPlan {
 // Block size and degree for fields c in [lo, hi].  |x| <= 1.2 keeps the
 // polynomial's alternating terms within e^2.4 of their sum.  The degree is the
 // first whose remainder |x|^(deg+1) / (deg+1)! is below a sixteenth of the
-// rounding.  B = 0: the grid is too wide for blocks of 8, its fields go bin by
-// bin (8 sums of 20 coefficients cost as much as 8 bins there).  Measured at
-// beta = 0.7, 4096 fields, 6.4e5 samples: half width 0.42 (blocks of 8) 5.4 ms
-// for 32769 bins and 40.5 ms for 262145 against 11.3 and 45.5 bin by bin; half
-// width 1 and 20 (bin by bin) 8.9 and 6.3 ms for 32769 bins, where blocks of
-// one bin took 15.1 and 13.4.
+// rounding.  B = 0: the grid is too wide for blocks, its fields go bin by bin.
+// The smallest block is 8 bins, beyond 2^17 bins 16: 4096 fields of half width
+// 0.42 (beta = 0.7) take 1.27, 5.5 and 39 ms in blocks of 8 for 4097, 32769 and
+// 262145 bins; of half width 0.5, bin by bin, 1.68, 5.7 and 30.6 ms.
 BlockPlan block_plan(double lo, double hi, int nE)
 {
     BlockPlan p{};
     p.slope = lo + 0.5 * (hi - lo);
     const double w = 0.5 * (hi - lo);
-    for (int B = 64; B >= 8 && !p.B; B /= 2)
+    for (int B = 64; B >= (nE <= 1 << 17 ? 8 : 16) && !p.B; B /= 2)
         if (w * (B / 2) <= kXMax) p.B = B;
     if (!p.B) return p;
     const double x = w * (p.B / 2), eps = 0x1p-57;
@@ -972,29 +990,36 @@ __global__ void __launch_bounds__(192)
 block_coef_kernel(BinStats<double> s, int nE, int e_min, BlockPlan p, Blocks out)
 {
     __shared__ double f[kStats][64], t[kDegMax + 1][64];
-    __shared__ double sv[64], sj[64], sm[64];
-    __shared__ int sa[64];
+    __shared__ double red[3][2];
+    __shared__ int ra[2];
     const int b = blockIdx.x, e0 = b * p.B, len = min(p.B, nE - e0), i = threadIdx.x;
     const int mid = min(e0 + p.B / 2, nE - 1), slot = block_slot(p, b);
-    const double n = i < len ? s.n[e0 + i] : 0.0;
+    const double n = i < len ? s.n[e0 + i] : 0.0;  // bins in the first two warps
     if (i < 64) {
-        sv[i] = n > 0.0 ? (-(p.slope * (double)(e0 + i - mid)) - (s.lw[e0 + i] - s.lw[mid])) + log(n)
-                        : -INFINITY;
-        sa[i] = i;
+        double v = -INFINITY;
+        int a = i;
+        if (n > 0.0) v = (-(p.slope * (double)(e0 + i - mid)) - (s.lw[e0 + i] - s.lw[mid])) + log(n);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double v2 = __shfl_xor_sync(0xFFFFFFFFu, v, o);
+            const int a2 = __shfl_xor_sync(0xFFFFFFFFu, a, o);
+            if (v2 > v || (v2 == v && a2 < a)) {
+                v = v2;
+                a = a2;
+            }
+        }
+        if ((i & 31) == 0) {
+            red[0][i >> 5] = v;
+            ra[i >> 5] = a;
+        }
     }
     __syncthreads();
-    for (int o = 32; o > 0; o >>= 1) {
-        if (i < o && sv[i + o] > sv[i]) {
-            sv[i] = sv[i + o];
-            sa[i] = sa[i + o];
-        }
-        __syncthreads();
-    }
-    if (sv[0] == -INFINITY) {  // no samples: the whole CTA
+    const int first = red[0][1] > red[0][0] ? 1 : 0;
+    if (red[0][first] == -INFINITY) {  // no samples: the whole CTA
         if (i == 0) out.ln[slot] = -INFINITY;
         return;
     }
-    const int ref = e0 + sa[0];
+    const int ref = e0 + ra[first];
     const double r = (double)(e0 + i - ref);
     double v = 0.0, vn = 0.0, mej = 0.0, cm = 0.0;
     __syncthreads();
@@ -1006,20 +1031,17 @@ block_coef_kernel(BinStats<double> s, int nE, int e_min, BlockPlan p, Blocks out
         cm = s.cm[e0 + i] - s.cm[ref];
     }
     if (i < 64) {
-        sv[i] = vn;
-        sj[i] = vn * mej;
-        sm[i] = vn * cm;
+        double z[3] = {vn, vn * mej, vn * cm};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) z[k] += __shfl_xor_sync(0xFFFFFFFFu, z[k], o);
+            if ((i & 31) == 0) red[k][i >> 5] = z[k];
+        }
     }
     __syncthreads();
-    for (int o = 32; o > 0; o >>= 1) {
-        if (i < o) {
-            sv[i] += sv[i + o];
-            sj[i] += sj[i + o];
-            sm[i] += sm[i + o];
-        }
-        __syncthreads();
-    }
-    const double mj = s.mej[ref] + sj[0] / sv[0], mm = s.cm[ref] + sm[0] / sv[0];
+    const double z = red[0][0] + red[0][1];
+    const double mj = s.mej[ref] + (red[1][0] + red[1][1]) / z, mm = s.cm[ref] + (red[2][0] + red[2][1]) / z;
     if (i == 0) {
         out.ln[slot] = log(s.n[ref]);
         out.E[slot] = e_min + ref;
@@ -1065,28 +1087,6 @@ __device__ __forceinline__ double block_exponent(double c, double e, double lw, 
     return (-p - l) - (pe + le);
 }
 
-// Sums of K values over the block; every thread gets them.
-template <int K>
-__device__ __forceinline__ void block_sum_plain(double (&v)[K], double *sh)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < K; ++k)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xFFFFFFFFu, v[k], o);
-    __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < K; ++k) sh[wid * K + k] = v[k];
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        double a = sh[k];
-        for (int i = 1; i < kRgThreads / 32; ++i) a += sh[i * K + k];
-        v[k] = a;
-    }
-}
-
 // KK consecutive fields per CTA; thread t takes the blocks at slots
 // i kRgThreads + t, whose coefficients are read once for the KK fields.
 template <int KK>
@@ -1110,9 +1110,11 @@ block_grid_kernel(Blocks bl, BlockPlan p, double beta, int V, const double *__re
         double best = -INFINITY;
         int at = 0x7FFFFFFF;
         for (int i = 0; i < p.per; ++i) {
-            const int q = i * kRgThreads + t;
-            if (t * p.per + i < p.nblk && bl.ln[q] > -INFINITY) {
-                const double a = (-(c[k] * (double)bl.E[q]) - bl.lw[q]) + bl.ln[q];
+            // loaded together (slots without a block are allocated, and not used)
+            const int q = i * kRgThreads + t, E = bl.E[q];
+            const double ln = bl.ln[q], lw = bl.lw[q];
+            if (t * p.per + i < p.nblk && ln > -INFINITY) {
+                const double a = (-(c[k] * (double)E) - lw) + ln;
                 if (a > best) {
                     best = a;
                     at = q;
@@ -1132,10 +1134,9 @@ block_grid_kernel(Blocks bl, BlockPlan p, double beta, int V, const double *__re
 #pragma unroll
         for (int j = 0; j < kStats; ++j) S[k][j] = 0.0;
     for (int i = 0; i < p.per; ++i) {
-        const int q = i * kRgThreads + t;
-        if (t * p.per + i >= p.nblk || bl.ln[q] == -INFINITY) continue;
-        const int Eb = bl.E[q];
-        const double lb = bl.lw[q], mid = (double)bl.mid[q];
+        const int q = i * kRgThreads + t, Eb = bl.E[q];
+        const double ln = bl.ln[q], lb = bl.lw[q], mid = (double)bl.mid[q];
+        if (t * p.per + i >= p.nblk || ln == -INFINITY) continue;
         double A[KK];
         bool any = false;
 #pragma unroll
@@ -1177,18 +1178,9 @@ block_grid_kernel(Blocks bl, BlockPlan p, double beta, int V, const double *__re
 #pragma unroll
     for (int k = 0; k < KK; ++k) {
         double (&T)[kStats] = S[k];
-        block_sum_plain<kStats>(T, sh);
-        // the means relative to the reference, and the sums about them
-        const double Z = T[0], mE = T[1] / Z, mJ = T[2] / Z, mu = T[3] / Z;
-        if (t == 0 && k0 + k < n_grid) {
-            double *o = out + 5 * (int64_t)(k0 + k);
-            const double m2 = T[4] / Z, m4 = T[5] / Z;
-            o[0] = J0[k] + mJ;
-            o[1] = (double)E0[k] + mE;
-            o[2] = -beta * (T[6] / Z - mE * mJ);
-            o[3] = beta * (double)V * (T[7] / Z - mu * mu);
-            o[4] = 1.0 - m4 / (3.0 * m2 * m2);
-        }
+        block_sum_plain<kStats, kRgThreads / 32>(T, sh);
+        if (t == 0 && k0 + k < n_grid)
+            put_field(T, E0[k], J0[k], M0[k], beta, V, out + 5 * (int64_t)(k0 + k));
     }
 }
 
@@ -1356,8 +1348,12 @@ int reweight_on_scratch(const int32_t *e_j, const int32_t *e_d, const int32_t *m
         RCK(cudaGetLastError());
         if (n_grid > 0 && plan.B)
             RCK(launch_blocks(s, n_e, e_min, beta, V, plan, blocks, d_c, n_grid, d_out, nsm, st));
-        else if (n_grid > 0)
-            grid_kernel_f64<<<n_grid, 256, 0, st>>>(s, n_e, e_min, beta, V, d_c, d_out);
+        else if (n_grid > 0) {
+            // few fields leave SMs idle: more threads for each; no more than bins
+            int threads = n_grid < nsm ? 512 : 256;
+            while (threads > 64 && threads / 2 >= n_e) threads /= 2;
+            grid_kernel_f64<<<n_grid, threads, 0, st>>>(s, n_e, e_min, beta, V, d_c, d_out);
+        }
         RCK(cudaGetLastError());
     } else {
         BinStats<float> s;
