@@ -10,8 +10,8 @@
 //      shifted by their maximum; C and chi are taken about the means, or about
 //      a bin that holds a good share of the weight, so no difference of large
 //      moments is ever formed.
-// Stage B runs in FP64 (blocks of bins), or in FP32 (bin by bin) where the
-// exponent -beta Delta_k E - lnW(E) is carried as a float pair (hi + lo,
+// Stage B runs in FP64 (blocks of bins, wide grids bin by bin), or in FP32 where
+// the exponent -beta Delta_k E - lnW(E) is carried as a float pair (hi + lo,
 // error-free products and sums) so that its O(10^5) magnitude does not eat the
 // 24-bit mantissa, and all sums are Kahan-compensated.
 #include <algorithm>
